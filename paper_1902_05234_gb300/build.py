@@ -65,12 +65,8 @@ def _compile(src: str, nvcc: str, debug: bool = False) -> str:
     elif src.endswith(".cu"):
         # every nvcc/cudafe/ptxas warning is an error: a host-only helper called
         # from device code is only a warning otherwise, and the kernel then
-        # silently compiles to nothing.  The bitsliced kernel (ct.cu) keeps 128
-        # plane registers per thread and runs at the 255-register limit with a
-        # few bytes of spill by design, so only it is exempt from the spill check.
-        cmd[1:1] = ["--Werror", "all-warnings"]
-        if os.path.basename(src) != "ct.cu":
-            cmd[1:1] = ["-Xptxas", "-warn-spills"]
+        # silently compiles to nothing.  Register spills count as warnings.
+        cmd[1:1] = ["--Werror", "all-warnings", "-Xptxas", "-warn-spills"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"compile failed: {' '.join(cmd)}\n{r.stdout}\n{r.stderr}")

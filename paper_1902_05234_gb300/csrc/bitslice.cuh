@@ -1,19 +1,23 @@
 // bitslice.cuh -- constant-time (table-free) AES on bit planes.
 //
-// 32 blocks are processed together: word W[c][p] holds, in bit j, bit p of
-// column c of block j (p = 8 r + b: row r, bit b of the byte).  Every step of
-// a round is then a fixed sequence of logic operations on these words, with no
-// memory access that depends on data -- the side channel the paper's remark on
-// xtime and power analysis (section 3.2.1, Def. 3) is about.  The logic comes
-// from the generated circuits of bitslice_circuits.h (see gen_bitslice.py),
-// each gate one LOP3:
-//   encryption round  S-box circuit per byte (the round key enters as the
-//                     circuit's output mask), ShiftRows as a permutation of
-//                     registers, MixColumns circuit per column;
-//   decryption round  InvShiftRows as a permutation, the inverse S-box's
-//                     nonlinear core per byte, then one circuit per column for
+// 8 blocks are processed together in 32 words: word W[p], p = 8 r + b, is the
+// plane of row r, bit b, and holds in bit 8 c + j that bit of the byte (r, c)
+// of block j -- byte c of the word is column c.  Every step of a round is then
+// a fixed sequence of logic operations on these words, with no memory access
+// that depends on data -- the side channel the paper's remark on xtime and
+// power analysis (section 3.2.1, Def. 3) is about.  The logic comes from the
+// generated circuits of bitslice_circuits.h (see gen_bitslice.py), each gate
+// one LOP3:
+//   encryption round  S-box circuit per row (the round key enters as the
+//                     circuit's output mask), ShiftRows as a byte rotation of
+//                     each word, one MixColumns circuit for the four columns;
+//   decryption round  InvShiftRows as byte rotations, the inverse S-box's
+//                     nonlinear core per row, then one circuit for
 //                     InvMixColumns of the S-box outputs plus the round key.
-// Round keys reach the circuits as mask planes (all-zero or all-one words)
+// With one word per (row, bit) the four columns share every gate, so 8 blocks
+// fill the words; the 24 rotations a round are all this costs against one
+// word per (column, row, bit) and 32 blocks, where ShiftRows is a renaming.
+// Round keys reach the circuits as mask planes (each byte all zeros or ones)
 // that the host derives from the schedule (see ct.cu): a key byte m wanted at
 // an S-box output enters the S-box's product chains as mu = OUT^-1 m, so it
 // costs no gate.  The functions are
@@ -206,107 +210,24 @@ static_assert(check_inv_mix_circuit(), "InvMixColumns output circuit");
 static_assert(check_mix_circuit(), "MixColumns circuit");
 
 // ------------------------------------------------------- rounds on planes
-// State: W[c][8 r + b] = plane (row r, column c, bit b).
+// State: W[8 r + b] = plane of row r, bit b; byte c of the word is column c,
+// bit j of that byte block j.
 struct Planes {
-    uint32_t w[4][32];
+    uint32_t w[32];
 };
 
 // Key planes of one step, in the state's layout: the key itself for step 0,
 // the mu planes (see ct.cu) for the rounds.
-struct RoundMasks {
-    uint32_t m[4][32];
+struct alignas(16) RoundMasks {
+    uint32_t m[32];
 };
 
 AESGB_HD void add_masks(Planes &s, const RoundMasks &k) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int p = 0; p < 32; ++p) s.w[c][p] ^= k.m[c][p];
+    for (int p = 0; p < 32; ++p) s.w[p] ^= k.m[p];
 }
 
-// Row r rotated left by r columns (ShiftRows, eq (19)) or right (inverse).
-template <int DIR>
-AESGB_HD void shift_rows(Planes &s) {
-#pragma unroll
-    for (int r = 1; r < 4; ++r)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            uint32_t t[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) t[c] = s.w[DIR == 0 ? (c + r) & 3 : (c - r + 4) & 3][8 * r + b];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) s.w[c][8 * r + b] = t[c];
-        }
-}
-
-// Encryption round: SubBytes with the folded key (as mu planes), ShiftRows,
-// and MixColumns unless it is the last round.
-template <bool MIX>
-AESGB_HD void enc_round(Planes &s, const RoundMasks &k) {
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int r = q & 3, c = q >> 2;
-        uint32_t in[16];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            in[b] = s.w[c][8 * r + b];
-            in[8 + b] = k.m[c][8 * r + b];
-        }
-        run<bsc::k_sbox_enc>(in, &s.w[c][8 * r]);
-    }
-    shift_rows<0>(s);
-    if (MIX)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) run<bsc::k_mix_columns>(s.w[c], s.w[c]);
-}
-
-// Decryption round: InvShiftRows, InvSubBytes, AddRoundKey and (unless it is
-// the last round) InvMixColumns, the last three per column: the S-box cores
-// take the key as mu planes, one circuit maps the column's four cores through
-// the S-box output map and InvMixColumns.
-template <bool MIX>
-AESGB_HD void dec_round(Planes &s, const RoundMasks &k) {
-    shift_rows<1>(s);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        uint32_t o[32];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            uint32_t in[16];
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                in[b] = s.w[c][8 * r + b];
-                in[8 + b] = k.m[c][8 * r + b];
-            }
-            run<bsc::k_sbox_core_dec>(in, &o[8 * r]);
-        }
-        if (MIX) {
-            run<bsc::k_inv_mix_out>(o, s.w[c]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; ++r) run<bsc::k_sbox_out_dec>(&o[8 * r], &s.w[c][8 * r]);
-        }
-    }
-}
-
-// The whole cipher on one 32-block plane set.  masks[0] is added first, then
-// round i = 1..nr uses masks[i] (host-built, see ct.cu).
-template <int DIR>
-AESGB_HD void cipher_planes(Planes &s, const RoundMasks *masks, int nr) {
-    add_masks(s, masks[0]);
-#pragma unroll 1
-    for (int i = 1; i < nr; ++i) {
-        if (DIR == 0) enc_round<true>(s, masks[i]);
-        else dec_round<true>(s, masks[i]);
-    }
-    if (DIR == 0) enc_round<false>(s, masks[nr]);
-    else dec_round<false>(s, masks[nr]);
-}
-
-// In-place transpose of a 32x32 bit matrix: afterwards bit j of a[i] is the
-// old bit i of a[j].  Five stages swap blocks of 16, 8, 4, 2, 1 bits between
-// words 16, 8, 4, 2, 1 apart; the 16- and 8-bit stages are byte permutes, the
-// others one shift (as a multiplication) and one bit-select per word.
+// Bytes of the 8-byte value y:x picked by the four nibbles of sel.
 AESGB_HD uint32_t byte_perm(uint32_t x, uint32_t y, uint32_t sel) {
 #if defined(__CUDA_ARCH__)
     return __byte_perm(x, y, sel);
@@ -318,9 +239,68 @@ AESGB_HD uint32_t byte_perm(uint32_t x, uint32_t y, uint32_t sel) {
 #endif
 }
 
-// x << s and x >> s (0 < s < 32) as multiplications, which the GPU runs on its
+// Row r rotated left by r columns (ShiftRows, eq (19)) or right (inverse):
+// column c is byte c, so the words of row r rotate by r bytes, one byte permute
+// each.  (As a multiplication and a multiply-add on the idle multiply pipe, two
+// instructions each, the whole cipher measured 2-3 % slower.)
+template <int DIR>
+AESGB_HD void shift_rows(Planes &s) {
+#pragma unroll
+    for (int r = 1; r < 4; ++r)
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            s.w[8 * r + b] = byte_perm(s.w[8 * r + b], 0u, r == 2 ? 0x1032u : (DIR == 0) == (r == 1) ? 0x0321u : 0x2103u);
+}
+
+// The whole cipher on one 8-block plane set.  masks[0] is added first, then
+// round i = 1..nr uses masks[i] (host-built, see ct.cu); the last round leaves
+// out (Inv)MixColumns.
+//   encryption  SubBytes with the folded key (as mu planes), ShiftRows,
+//               MixColumns;
+//   decryption  InvShiftRows, then InvSubBytes, AddRoundKey and InvMixColumns:
+//               the S-box cores take the key as mu planes, one circuit maps the
+//               four rows' cores through the S-box output map and InvMixColumns.
+// One loop serves all rounds, the last leaving from its middle: a second copy
+// of the last round in the instruction stream measured 0.3-0.6 % slower at
+// 1 GiB, two rounds per iteration 2-3 % slower.
+template <int DIR>
+AESGB_HD void cipher_planes(Planes &s, const RoundMasks *masks, int nr) {
+    add_masks(s, masks[0]);
+#pragma unroll 1
+    for (int i = 1;; ++i) {
+        uint32_t o[32];
+        if (DIR == 1) shift_rows<1>(s);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            uint32_t in[16];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                in[b] = s.w[8 * r + b];
+                in[8 + b] = masks[i].m[8 * r + b];
+            }
+            if (DIR == 0) run<bsc::k_sbox_enc>(in, &s.w[8 * r]);
+            else run<bsc::k_sbox_core_dec>(in, &o[8 * r]);
+        }
+        if (DIR == 0) shift_rows<0>(s);
+        if (i == nr) {
+            if (DIR == 1)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) run<bsc::k_sbox_out_dec>(&o[8 * r], &s.w[8 * r]);
+            return;
+        }
+        if (DIR == 0) run<bsc::k_mix_columns>(s.w, s.w);
+        else run<bsc::k_inv_mix_out>(o, s.w);
+    }
+}
+
+// In-place transpose of a 32x32 bit matrix: afterwards bit j of a[i] is the
+// old bit i of a[j].  Five stages swap blocks of 16, 8, 4, 2, 1 bits between
+// words 16, 8, 4, 2, 1 apart; the 16- and 8-bit stages are byte permutes, the
+// others one shift and one bit-select per word.
+//
+// x << s (0 < s < 32) as a multiplication, which the GPU runs on its
 // multiply-add pipe rather than the integer-logic pipe that the circuits keep
-// busy: x * 2^s keeps the low word, the high word of x * 2^(32-s) is x >> s.
+// busy.  (x >> s as the high word of a product gains nothing.)
 AESGB_HD uint32_t shl_mul(uint32_t x, int s) {
 #if defined(__CUDA_ARCH__)
     uint32_t d;
@@ -328,13 +308,6 @@ AESGB_HD uint32_t shl_mul(uint32_t x, int s) {
     return d;
 #else
     return x << s;
-#endif
-}
-AESGB_HD uint32_t shr_mul(uint32_t x, int s) {
-#if defined(__CUDA_ARCH__)
-    return __umulhi(x, 1u << (32 - s));
-#else
-    return x >> s;
 #endif
 }
 
@@ -360,7 +333,7 @@ AESGB_HD void transpose32(uint32_t *a) {
             if (k & s) continue;  // k runs over the words whose partner is k + s
             const uint32_t x = a[k], y = a[k + s];
             a[k] = lop3<0xD8>(x, shl_mul(y, s), ~m);     // ~m ? (y << s) : x
-            a[k + s] = lop3<0xD8>(y, shr_mul(x, s), m);  //  m ? (x >> s) : y
+            a[k + s] = lop3<0xD8>(y, x >> s, m);         //  m ? (x >> s) : y
         }
     }
 }

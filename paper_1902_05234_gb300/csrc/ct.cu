@@ -1,13 +1,14 @@
 // ct.cu -- constant-time ECB: the bitsliced cipher of bitslice.cuh on GB300.
 //
-// Each thread owns 32 blocks: lane l of a warp takes blocks base + 32 j + l,
-// j = 0..31, so every warp-wide 128-bit load or store still covers 512
-// contiguous bytes.  The thread transposes its 32 x 128 bits into 128 bit
-// planes, runs the rounds as logic operations on whole planes, transposes
-// back and stores.  No address depends on key or data.  Round keys reach the
-// circuits as mask planes built on the host from the schedule (one mask byte
-// per byte position and key step, see build_masks) and expanded into shared
-// memory at the start of the kernel.
+// Each thread owns 8 blocks at a time: lane l of a warp takes blocks base +
+// 32 j + l, j = 0..7, so every warp-wide 128-bit load or store still covers
+// 512 contiguous bytes.  The thread transposes its 32 words into 32 bit planes
+// (word 8 c + j, column c of block j, becomes bit 8 c + j of every plane), runs
+// the rounds as logic operations on whole planes, transposes back and stores.
+// No address depends on key or data.  Round keys reach the circuits as mask
+// planes built on the host from the schedule (one mask byte per byte position
+// and key step, see build_masks) and expanded into shared memory at the start
+// of the kernel.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -20,7 +21,8 @@
 
 namespace aesgb {
 
-constexpr int kCtThreads = 256;  // 128 plane registers + the circuits' temporaries per thread
+constexpr int kCtThreads = 512;  // largest CTA (95 registers: one per SM)
+constexpr int kCtBlocks = 8;  // AES blocks per thread and pass: one word per (row, bit) plane
 
 struct CtArgs {
     const uint4 *in;
@@ -44,79 +46,109 @@ struct CtArgs {
 //   decryption  (inverse cipher, FIPS-197 5.3): step 0 is K_Nr; round i adds
 //               K_{Nr-i} right after InvSubBytes, m = K_{Nr-i}, and the column
 //               circuit applies InvMixColumns to the sum.
+struct MuTables {
+    uint8_t of[2][256];  // OUT^-1 m of the encryption and of the decryption S-box circuit
+};
+constexpr MuTables make_mu_tables() {
+    MuTables t{};
+    for (int m = 0; m < 256; ++m) {
+        t.of[0][m] = bs::apply_rows(bsc::k_mu_enc, static_cast<uint8_t>(m));
+        t.of[1][m] = bs::apply_rows(bsc::k_mu_dec, static_cast<uint8_t>(m));
+    }
+    return t;
+}
+constexpr MuTables kMu = make_mu_tables();
+
+// MixColumns / InvMixColumns of one key column on the host, from the round
+// tables: te0[x] is the MixColumns column of S(x) in row 0 (eq (22)), td0[x]
+// the InvMixColumns column of InvS(x); rows 1..3 are byte rotations.
+uint32_t key_column(const uint32_t (&tab)[256], const uint8_t (&undo)[256], const uint8_t *k) {
+    uint32_t v = 0;
+    for (int r = 0; r < 4; ++r) {
+        const uint32_t t = tab[undo[k[r]]];
+        v ^= r == 0 ? t : (t << (8 * r)) | (t >> (32 - 8 * r));
+    }
+    return v;
+}
+
 void build_masks(int dir, const uint32_t *rk, int nr, uint8_t (*out)[16]) {
     uint8_t w[240];
     std::memcpy(w, rk, 16 * (nr + 1));
-    if (dir == 1)  // rk is dw: its keys 1..Nr-1 are InvMixColumns(w_r); MixColumns gives w back
-        for (int r = 1; r < nr; ++r)
-            for (int c = 0; c < 4; ++c) {
-                uint32_t col;
-                std::memcpy(&col, w + 16 * r + 4 * c, 4);
-                col = bsmath::mix_column_model(col);
-                std::memcpy(w + 16 * r + 4 * c, &col, 4);
-            }
-    std::memcpy(out[0], w + (dir == 0 ? 0 : 16 * nr), 16);
-    for (int i = 1; i <= nr; ++i) {
-        uint8_t m[16];
-        if (dir == 0) {
-            uint8_t k[16];
-            for (int c = 0; c < 4; ++c) {
-                uint32_t col;
-                std::memcpy(&col, w + 16 * i + 4 * c, 4);
-                if (i < nr) col = bsmath::inv_mix_column_model(col);
-                std::memcpy(k + 4 * c, &col, 4);
-            }
-            for (int q = 0; q < 16; ++q) {
-                const int r = q & 3, c = q >> 2;
-                m[q] = static_cast<uint8_t>(0x63 ^ k[r + 4 * ((c - r + 4) & 3)]);
-            }
-        } else {
-            std::memcpy(m, w + 16 * (nr - i), 16);
-        }
-        for (int q = 0; q < 16; ++q) out[i][q] = bs::apply_rows(dir == 0 ? bsc::k_mu_enc : bsc::k_mu_dec, m[q]);
+    // encryption needs InvMixColumns of keys 1..Nr-1; dw (decryption) holds
+    // InvMixColumns(w_r) there, and MixColumns gives w back
+    uint8_t mixed[240];
+    for (int q = 16; q < 16 * nr; q += 4) {
+        const uint32_t col = dir == 0 ? key_column(kAes.td0, kAes.sbox, w + q) : key_column(kAes.te0, kAes.isbox, w + q);
+        std::memcpy(mixed + q, &col, 4);
     }
+    std::memcpy(mixed, w, 16);
+    std::memcpy(mixed + 16 * nr, w + 16 * nr, 16);
+    std::memcpy(out[0], mixed + (dir == 0 ? 0 : 16 * nr), 16);
+    for (int i = 1; i <= nr; ++i)
+        for (int q = 0; q < 16; ++q) {
+            const int r = q & 3, c = q >> 2;
+            const uint8_t m = dir == 0 ? static_cast<uint8_t>(0x63 ^ mixed[16 * i + r + 4 * ((c - r + 4) & 3)])
+                                       : mixed[16 * (nr - i) + q];
+            out[i][q] = kMu.of[dir][m];
+        }
 }
 
-// Mask byte -> 8 planes, in the state's layout (plane 8r + b of column c).
+// Mask bytes -> planes, in the state's layout: plane p = 8 r + b of step i / 32,
+// byte c all ones where bit b of the mask byte (r, c) is set.
 AESGB_HD void expand_mask(const uint8_t (*m)[16], int i, bs::RoundMasks *dst) {
-    const int app = i >> 7, p = i & 127, c = p >> 5, rb = p & 31;
+    const int app = i >> 5, p = i & 31, r = p >> 3, b = p & 7;
 #if defined(__CUDA_ARCH__)
     if (!AESGB_CHECK(app < 15)) return;
 #endif
-    dst[app].m[c][rb] = ((m[app][(rb >> 3) + 4 * c] >> (rb & 7)) & 1) ? 0xffffffffu : 0u;
+    uint32_t v = 0;
+    for (int c = 0; c < 4; ++c) v |= ((m[app][r + 4 * c] >> b) & 1u) * (0xffu << (8 * c));
+    dst[app].m[p] = v;
 }
 
+// Bound: the integer-logic (ALU) pipe, 64 lanes per clock per SM: 527 counted
+// operations per block for AES-128 encryption (aes_ct_ops_per_block), 30 byte
+// permutes for ShiftRows and about 10 more for addresses and bounds.  A unit of
+// work is a warp's 256 blocks (4 KiB).  8 blocks and 32 planes per thread take
+// 95 registers without spill; the form with 32 blocks and 128 planes, one word
+// per (column, row, bit), needs no permutes but 255 registers and a unit of
+// 16 KiB, so a pass was four times as long and a 1 MiB buffer filled 8 SMs.
+// Units go round the CTAs first and then the warps of each, so that every SM,
+// and every quarter of one, gets the same number within one.  Measured against
+// that form (a replayed graph of launches, AES-128 encryption): 4 KiB 20.1 ->
+// 5.9 us, 1 MiB 36.2 -> 5.9 us, 16 MiB 37.9 -> 33.4 us, 1 GiB 4,345 -> 4,394
+// Gbit/s; AES-256 decryption of 256 MiB 2,853 -> 3,019 Gbit/s.
 template <int DIR>
 __global__ void __launch_bounds__(kCtThreads, 1) ct_kernel(const __grid_constant__ CtArgs a) {
     __shared__ bs::RoundMasks masks[15];
-    for (int i = threadIdx.x; i < (a.nr + 1) * 128; i += blockDim.x) expand_mask(a.masks, i, masks);
+    for (int i = threadIdx.x; i < (a.nr + 1) * 32; i += blockDim.x) expand_mask(a.masks, i, masks);
     __syncthreads();
     griddep_release();
     griddep_wait();  // global memory only after this (see aes_kernels.cuh)
     const uint32_t lane = threadIdx.x & 31u;
+    constexpr unsigned long long kUnit = 32ull * kCtBlocks;  // blocks of a warp's pass
     const unsigned long long wpc = blockDim.x >> 5;
-    const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * wpc * 1024ull;
+    const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * wpc * kUnit;
     const unsigned long long n = a.nblocks;
-    for (unsigned long long base = (blockIdx.x * wpc + (threadIdx.x >> 5)) * 1024ull; base < n; base += step) {
+    // units go round the CTAs first, then the warps of each
+    for (unsigned long long base = (static_cast<unsigned long long>(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * kUnit;
+         base < n; base += step) {
         bs::Planes s;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < kCtBlocks; ++j) {
             const unsigned long long blk = base + 32ull * j + lane;
             const uint4 v = blk < n ? ld_block(a.in + blk) : make_uint4(0, 0, 0, 0);
-            s.w[0][j] = v.x;
-            s.w[1][j] = v.y;
-            s.w[2][j] = v.z;
-            s.w[3][j] = v.w;
+            s.w[j] = v.x;
+            s.w[8 + j] = v.y;
+            s.w[16 + j] = v.z;
+            s.w[24 + j] = v.w;
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) bs::transpose32(s.w[c]);
+        bs::transpose32(s.w);
         bs::cipher_planes<DIR>(s, masks, a.nr);
+        bs::transpose32(s.w);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) bs::transpose32(s.w[c]);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < kCtBlocks; ++j) {
             const unsigned long long blk = base + 32ull * j + lane;
-            if (blk < n) st_block(a.out + blk, make_uint4(s.w[0][j], s.w[1][j], s.w[2][j], s.w[3][j]));
+            if (blk < n) st_block(a.out + blk, make_uint4(s.w[j], s.w[8 + j], s.w[16 + j], s.w[24 + j]));
         }
     }
 }
@@ -149,29 +181,37 @@ int aes_ecb_crypt_ct(int dir, const uint32_t *rk, int nrounds, const uint8_t *in
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
     const void *fn = dir == 0 ? reinterpret_cast<const void *>(&ct_kernel<0>)
                               : reinterpret_cast<const void *>(&ct_kernel<1>);
-    aes_launch_cfg c{kCtThreads, 1, 0, 0};
-    int grid = 0;
-    st = persistent_grid(fn, dev, c, 0, static_cast<unsigned long long>(kCtThreads) * 32ull, nblocks, &grid,
-                         nullptr);
-    if (st != AES_OK) return st;
+    const int sms = sm_count(dev);
+    if (sms < 0) return sms;
+    // One CTA per SM, or one per unit when there are fewer.  One warp per SM
+    // quarter keeps the ALU pipe 94 % busy (its circuits are independent), so a
+    // buffer with few units per SM gets a small CTA, whose registers leave room
+    // for the next launch's to start behind it (programmatic dependent launch);
+    // large buffers get 16 warps, which run closely enough together to share the
+    // instruction cache: 256 MiB, AES-128 encryption, took 492.7 us with 512
+    // threads, 502.1 with 256, 507.2 with five CTAs of 128.
+    const unsigned long long units = (nblocks + 32 * kCtBlocks - 1) / (32 * kCtBlocks);
+    const unsigned long long per_sm = (units + sms - 1) / sms;
+    const int threads = per_sm > 8 ? kCtThreads : per_sm > 4 ? 256 : 128;
+    const int grid = static_cast<int>(units < static_cast<unsigned long long>(sms) ? units : sms);
     void *params[] = {&args};
-    return launch_pdl(fn, grid, kCtThreads, 0, params, stream);
+    return launch_pdl(fn, grid, threads, 0, params, stream);
 }
 
 int aes_ct_ops_per_block(int dir, int nrounds, double *ops_per_block) {
     if ((dir != 0 && dir != 1) || !ops_per_block) return AES_E_ARG;
     const int st = check_nrounds(nrounds);
     if (st != AES_OK) return st;
-    // per thread and 32-block group: 128 planes of step-0 key, the rounds,
-    // 8 transposes of 32 words (stages 16 and 8: one byte permute per word,
+    // per thread and 8-block group: 32 planes of step-0 key, the rounds, 2
+    // transposes of 32 words (stages 16 and 8: one byte permute per word,
     // stages 4, 2 and 1: one bit-select per word)
-    long long g = 128 + 8 * (2 * 32 + 3 * 32);
+    long long g = 32 + 2 * (2 * 32 + 3 * 32);
     if (dir == 0)
-        g += 16LL * nrounds * bsc::k_sbox_enc.kGates + 4LL * (nrounds - 1) * bsc::k_mix_columns.kGates;
+        g += 4LL * nrounds * bsc::k_sbox_enc.kGates + (nrounds - 1LL) * bsc::k_mix_columns.kGates;
     else
-        g += 16LL * nrounds * bsc::k_sbox_core_dec.kGates + 4LL * (nrounds - 1) * bsc::k_inv_mix_out.kGates +
-             16LL * bsc::k_sbox_out_dec.kGates;
-    *ops_per_block = static_cast<double>(g) / 32.0;
+        g += 4LL * nrounds * bsc::k_sbox_core_dec.kGates + (nrounds - 1LL) * bsc::k_inv_mix_out.kGates +
+             4LL * bsc::k_sbox_out_dec.kGates;
+    *ops_per_block = static_cast<double>(g) / kCtBlocks;
     return AES_OK;
 }
 
@@ -182,22 +222,23 @@ int aes_ct_selftest_host(int dir, const uint32_t *rk, int nrounds, const uint8_t
     if (st != AES_OK) return st;
     uint8_t mb[15][16];
     build_masks(dir, rk, nrounds, mb);
-    static bs::RoundMasks masks[15];  // 7.5 KB: kept off the host stack
-    for (int i = 0; i < (nrounds + 1) * 128; ++i) expand_mask(mb, i, masks);
-    for (size_t g = 0; g < nblocks; g += 32) {
+    bs::RoundMasks masks[15];
+    for (int i = 0; i < (nrounds + 1) * 32; ++i) expand_mask(mb, i, masks);
+    for (size_t g = 0; g < nblocks; g += kCtBlocks) {
         bs::Planes s;
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < kCtBlocks; ++j) {
             uint32_t v[4] = {0, 0, 0, 0};
             if (g + j < nblocks) std::memcpy(v, in + 16 * (g + j), 16);
-            for (int c = 0; c < 4; ++c) s.w[c][j] = v[c];
+            for (int c = 0; c < 4; ++c) s.w[8 * c + j] = v[c];
         }
-        for (int c = 0; c < 4; ++c) bs::transpose32(s.w[c]);
+        bs::transpose32(s.w);
         if (dir == 0) bs::cipher_planes<0>(s, masks, nrounds);
         else bs::cipher_planes<1>(s, masks, nrounds);
-        for (int c = 0; c < 4; ++c) bs::transpose32(s.w[c]);
-        for (int j = 0; j < 32; ++j) {
+        bs::transpose32(s.w);
+        for (int j = 0; j < kCtBlocks; ++j) {
             if (g + j >= nblocks) break;
-            uint32_t v[4] = {s.w[0][j], s.w[1][j], s.w[2][j], s.w[3][j]};
+            uint32_t v[4];
+            for (int c = 0; c < 4; ++c) v[c] = s.w[8 * c + j];
             std::memcpy(out + 16 * (g + j), v, 16);
         }
     }

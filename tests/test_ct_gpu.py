@@ -1,6 +1,6 @@
 """Constant-time (bitsliced) ECB on the GPU: bit-exact against the oracle
-for every key size and direction, ragged sizes that leave partial 32-block
-groups and partial warp chunks, and equal to the T-table path on a larger
+for every key size and direction, ragged sizes that leave partial 8-block
+groups and partial warp units, and equal to the T-table path on a larger
 buffer."""
 import numpy as np
 import pytest
@@ -67,3 +67,24 @@ def test_logic_rate_calibration():
     assert 16 < per_sm_per_clk <= 64 * 1.05, per_sm_per_clk
     with pytest.raises(aesgb.AesError):
         aesgb.aes_calibrate_logic_rate(sink, 16)
+
+
+@pytest.mark.parametrize("units_per_sm", [0, 4, 8, 17])
+def test_ct_unit_and_cta_size_edges(orc, units_per_sm):
+    """A warp's unit is 256 blocks and 8 blocks share a thread's words; the CTA
+    size changes above 4 and 8 units per SM, and above 16 the warps take a
+    second unit: one block below, at and above each of those."""
+    torch = torch_cuda()
+    edge = max(256, 256 * units_per_sm * aesgb.aes_device_sm_count(0))
+    key = wl.random_key(256, 223).tobytes()
+    enc, dec, nr = aesgb.aes_expand_key(256, key)
+    for n in (7, 8, 9) * (units_per_sm == 0) + (edge - 1, edge, edge + 1):
+        data = wl.random_bytes(16 * n, 224 + n)
+        x = torch.from_numpy(data).cuda()
+        y = torch.full((16 * n + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+        for direction, rk in ((0, enc), (1, dec)):
+            aesgb.aes_ecb_crypt_ct(direction, rk, nr, x, y, n)
+            torch.cuda.synchronize()
+            got = y.cpu().numpy()
+            assert np.array_equal(got[:16 * n], orc.ecb(direction, key, data, nthreads=8)), (n, direction)
+            assert np.all(got[16 * n:] == 0x5A)
