@@ -205,25 +205,34 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 
 }  // namespace
 
-// Untuned choice: R4 tables, 2 blocks per thread and 1,024 threads when the
-// buffer fills every SM several times over; smaller buffers get R2 tables,
-// 2 blocks per thread and 256 threads with as many CTAs per SM as fit (three):
-// small CTAs spread a small buffer over every SM, and CTAs that finish early
-// make room for the next launch's CTAs to fill their tables.
-aes_launch_cfg default_cfg(int /*dir*/, int /*nrounds*/, size_t nblocks) {
+// Untuned choice, by blocks per SM.  From 1,024 up one CTA of 1,024 threads per
+// SM, one block per thread: 32 warps keep the data pipe full and the unit of
+// 512 bytes divides evenly.  R4 tables encrypt; R2 decrypts, whose 128 KiB fill
+// faster than R4's 160, up to 16,384, from where the fill does not count.
+// From 128 up R2, 512 threads, as many CTAs as fit; below that 256 threads x 2
+// blocks: few, small CTAs, so that a stream of short launches finds room.
+// Replayed graph, against 256 threads x 2 blocks up to 16,384 blocks per SM:
+//   AES-128 encryption  2 MiB 5.4 -> 4.2 us, 4 MiB 7.1 -> 6.4, 16 MiB 21.0 ->
+//   19.65, 32 MiB 38.8 -> 37.5; 128 MiB (2 blocks per thread) 145.5 -> 144.9
+//   AES-256 decryption  4 MiB 8.8 -> 8.6 us, 16 MiB 27.8 -> 26.9, 32 MiB 52.2 -> 51.6
+aes_launch_cfg default_cfg(int dir, int /*nrounds*/, size_t nblocks) {
+    const int found = current_sms();
+    const size_t sms = static_cast<size_t>(found > 0 ? found : 152);
     aes_launch_cfg c;
-    c.ctas_per_sm = 1;
-    const size_t sms = static_cast<size_t>(current_sms() > 0 ? current_sms() : 152);
-    if (nblocks >= sms * 16384) {
-        c.layout = AES_LAYOUT_R4;
+    c.blocks_per_thread = 1;
+    if (nblocks >= sms * 1024) {
+        c.layout = dir == 0 || nblocks >= sms * 16384 ? AES_LAYOUT_R4 : AES_LAYOUT_R2;
         c.threads = 1024;
-        c.blocks_per_thread = 2;
+        c.ctas_per_sm = 1;
         return c;
     }
     c.layout = AES_LAYOUT_R2;
-    c.threads = 256;
-    c.blocks_per_thread = 2;
+    c.threads = 512;
     c.ctas_per_sm = 0;
+    if (nblocks < sms * 128) {
+        c.threads = 256;
+        c.blocks_per_thread = 2;
+    }
     return c;
 }
 

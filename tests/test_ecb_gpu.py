@@ -330,3 +330,19 @@ def test_even_shares_at_one_cta_per_sm(orc, direction):
             assert ok and np.array_equal(got, exp), (nb, n)
             got, ok = gpu_ecb(direction, key, data, cfg=cfg, inplace=True, guard=64)
             assert ok and np.array_equal(got, exp), (nb, n, "in place")
+
+
+@pytest.mark.parametrize("blocks_per_sm", [128, 1024])
+def test_default_cfg_small_size_switches(orc, blocks_per_sm):
+    """The other two lines of the untuned choice (256 threads x 2 blocks, 512
+    threads, 1,024 threads): buffers just below, at and above each, both
+    directions, in units that go round the CTAs with a ragged last one."""
+    torch = torch_cuda()
+    edge = aesgb.aes_device_sm_count(torch.cuda.current_device()) * blocks_per_sm
+    key = wl.random_key(192, 14).tobytes()
+    for n in (edge - 1, edge, edge + 33):
+        data = wl.random_bytes(16 * n, 15)
+        for direction in (0, 1):
+            cfg = aesgb.aes_ecb_get_cfg(direction, 12, n)
+            got, ok = gpu_ecb(direction, key, data, guard=64)
+            assert ok and np.array_equal(got, orc.ecb(direction, key, data, nthreads=16)), (n, direction, cfg)
