@@ -376,6 +376,25 @@ struct ParamKey {
     __device__ __forceinline__ uint32_t operator()(int i) const { return w[i]; }
 };
 
+// Table t at byte b of word s, for layouts that keep only T0 and T1 too (one
+// column's worth at a time; full_round rotates the pair T2 ^ T3 once).
+template <class TabT>
+__device__ __forceinline__ uint32_t lookup_t(const TabT &tab, int t, uint32_t s, int b) {
+    const uint32_t v = tab.lookup(t, s, b);
+    return pair_rotate<TabT>() && t >= 2 ? __byte_perm(v, 0u, 0x1032u) : v;
+}
+
+// Rounds R0..NR on NB states.
+template <int DIR, int NR, int NB, int R0, class TabT, class Key>
+__device__ __forceinline__ void cipher_rounds(const TabT &tab, const Key &k, uint32_t (&s)[NB][4]) {
+#pragma unroll
+    for (int r = R0; r < NR; ++r)
+#pragma unroll
+        for (int i = 0; i < NB; ++i) full_round<DIR>(tab, s[i], k, 4 * r);
+#pragma unroll
+    for (int i = 0; i < NB; ++i) final_round<DIR>(tab, s[i], k, 4 * NR);
+}
+
 // Full cipher (encrypt) or equivalent inverse cipher (decrypt) on NB states.
 template <int DIR, int NR, int NB, class TabT, class Key>
 __device__ __forceinline__ void cipher_states(const TabT &tab, const Key &k, uint32_t (&s)[NB][4]) {
@@ -383,12 +402,7 @@ __device__ __forceinline__ void cipher_states(const TabT &tab, const Key &k, uin
     for (int i = 0; i < NB; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) s[i][j] ^= k(j);
-#pragma unroll
-    for (int r = 1; r < NR; ++r)
-#pragma unroll
-        for (int i = 0; i < NB; ++i) full_round<DIR>(tab, s[i], k, 4 * r);
-#pragma unroll
-    for (int i = 0; i < NB; ++i) final_round<DIR>(tab, s[i], k, 4 * NR);
+    cipher_rounds<DIR, NR, NB, 1>(tab, k, s);
 }
 
 // Programmatic dependent launch.  The host launches the single-buffer kernels

@@ -141,3 +141,62 @@ def test_cfb_roundtrip_with_oracle_encryption(orc):
     aesgb.aes_cfb_decrypt(enc, nr, iv, x, y, pt.size // 16)
     torch.cuda.synchronize()
     assert np.array_equal(y.cpu().numpy(), pt)
+
+
+@pytest.mark.parametrize("passes", [1, 2, 4, 8, 9, 33])
+def test_ctr_units_start_anywhere_in_a_group(orc, passes):
+    """The CTR kernel shares the first two rounds inside groups of 256 counter
+    blocks and cuts them into units of 1, 2, 4 or 8 passes by the buffer's size:
+    sizes at the edge of each choice, counters that start at the first, second,
+    middle and last block of a group, and one whose carry leaves the lower 64 bits."""
+    torch = torch_cuda()
+    key = wl.random_key(256, 96).tobytes()
+    enc, _, nr = aesgb.aes_expand_key(256, key)
+    n = aesgb.aes_device_sm_count(torch.cuda.current_device()) * 1024 * passes + 1
+    data = wl.random_bytes(16 * n, 96)
+    x = torch.from_numpy(data).cuda()
+    y = torch.full((16 * n + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    for last, carry in ((0, False), (1, False), (128, False), (255, False), (255, True)):
+        if passes > 9 and last not in (1, 255):
+            continue                                      # 80 MB: two of them
+        ctr0 = np.full(16, 0xFF if carry else 0x37, np.uint8)
+        ctr0[0], ctr0[15] = 0x11, last
+        aesgb.aes_ctr_crypt(enc, nr, ctr0, x, y, n)
+        torch.cuda.synchronize()
+        got = y.cpu().numpy()
+        assert np.all(got[16 * n:] == 0x5A)
+        # the oracle on the first and last 3,000 blocks (counter + block index)
+        for first in (0, n - 3000):
+            c = (int.from_bytes(ctr0.tobytes(), "big") + first) % (1 << 128)
+            part = slice(16 * first, 16 * (first + 3000))
+            assert np.array_equal(got[part], orc.ctr(key, np.frombuffer(c.to_bytes(16, "big"), np.uint8),
+                                                     data[part])), (n, last, carry, first)
+        # and everything between: CTR is its own inverse, and ECB encryption of
+        # the counter blocks through the table path gives the same key stream
+        z = torch.empty(16 * n, dtype=torch.uint8, device="cuda")
+        big = int.from_bytes(ctr0.tobytes(), "big")
+        hi, lo = big >> 64, big & ((1 << 64) - 1)
+        low = (np.arange(n, dtype=np.uint64) + np.uint64(lo)).astype(np.uint64)
+        high = np.uint64(hi) + (low < np.uint64(lo)).astype(np.uint64)
+        blocks = np.stack([high, low], 1).astype(">u8").view(np.uint8).reshape(-1)
+        ctrs = torch.from_numpy(blocks.copy()).cuda()
+        aesgb.aes_ecb_encrypt(enc, nr, ctrs, z, n)
+        assert torch.equal(z ^ x, y[:16 * n]), (n, last, carry)
+
+
+@pytest.mark.parametrize("more", [-1, 0, 33])
+def test_chained_modes_at_the_size_switch(orc, more):
+    """CBC and CFB decryption change their launch shape at 1,024 blocks per SM."""
+    torch = torch_cuda()
+    n = aesgb.aes_device_sm_count(torch.cuda.current_device()) * 1024 + more
+    key = wl.random_key(192, 97).tobytes()
+    enc, dec, nr = aesgb.aes_expand_key(192, key)
+    data = wl.random_bytes(16 * n, 97)
+    iv = wl.random_bytes(16, 98)
+    x = torch.from_numpy(data).cuda()
+    y = torch.full((16 * n + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+    for call, rk, ref in ((aesgb.aes_cbc_decrypt, dec, orc.cbc_decrypt), (aesgb.aes_cfb_decrypt, enc, orc.cfb_decrypt)):
+        call(rk, nr, iv, x, y, n)
+        torch.cuda.synchronize()
+        got = y.cpu().numpy()
+        assert np.array_equal(got[:16 * n], ref(key, iv, data)) and np.all(got[16 * n:] == 0x5A), (call.__name__, n)
