@@ -106,9 +106,10 @@ int aes_debug_bounds_violations(unsigned long long *count);
  * disarms it.  AES_E_ARG if either is negative.  Process-wide. */
 int aes_test_fail_allocs(int skip, int count);
 
-/* Debug build only: exactly-once coverage of the batch kernel's work counter.
- * Each chunk (chunk_blocks consecutive blocks of one message, the unit a warp
- * takes from the counter) adds one to its tag, for chunk indices below 65,536.
+/* Debug build only: exactly-once coverage of the batch kernel's work.
+ * Each chunk (chunk_blocks consecutive blocks of one message, from its start)
+ * adds one to its tag in the warp that takes its first pass, for chunk indices
+ * below 65,536.
  * Returns, over all batch launches since the last call: *once the chunks
  * tagged exactly once, *repeated those tagged more than once, *beyond the
  * chunks whose index lies past the tags; then clears the tags.  After ONE
@@ -245,27 +246,29 @@ typedef struct aes_desc {
 typedef struct aes_batch_cfg {
     int32_t threads;           /* threads per CTA (multiple of 32, <= 512: keys sit in registers)    */
     int32_t blocks_per_thread; /* 1, 2 or 4                                                           */
-    int32_t chunk_passes;      /* a warp's unit of work = 32 * blocks_per_thread * chunk_passes blocks */
+    int32_t chunk_passes;      /* a chunk is 32 * blocks_per_thread * chunk_passes blocks of a message;
+                                  a warp's share of work at a time is at most two of them          */
     int32_t ctas_per_sm;       /* 0 or 1 (the tables take most of the shared memory)                */
     int32_t layout_enc;        /* table layout of the encryption phase and of the decryption      */
-    int32_t layout_dec;        /* phase (aes_layout; section 4.2): the pairs R4/R2 (the default,
-                                  blocks_per_thread 1, 2 or 4), R4/R4, R2/R2 and R1/R1 (1 or 2);
-                                  another pair is AES_E_CONFIG                                       */
+    int32_t layout_dec;        /* phase (aes_layout; section 4.2): the pairs R4/R2
+                                  (blocks_per_thread 1, 2 or 4), R4/R4 (the default), R2/R2 and
+                                  R1/R1 (1 or 2); another pair is AES_E_CONFIG                       */
 } aes_batch_cfg;
 
 /* Bytes of DEVICE workspace a batch of n descriptors needs (plan header, the
- * message order and the chunk prefix: about 20 bytes per descriptor). */
+ * message order and the cost prefix: about 20 bytes per descriptor). */
 size_t aes_batch_workspace_bytes(int n);
 
 /* Most descriptors one batch call takes (AES_E_RANGE above it, nothing queued). */
 #define AES_BATCH_MAX_DESCS (1 << 28)
 
 /* Batched ECB with a caller-owned workspace.  Enqueues two kernels on
- * `stream`: a one-CTA plan kernel (validation, encryptions-first order, chunk
- * prefix) and the persistent batch kernel (one CTA per SM; each warp takes
- * the next chunk from an atomic work counter, finds the chunk's message by a
- * warp-wide 32-ary search of the prefix and stages its round keys through
- * shared memory into registers).  Allocates nothing and never synchronises,
+ * `stream`, three above 1,024 descriptors: the plan (validation,
+ * encryptions-first order, prefix of the messages' costs) and the persistent
+ * batch kernel (one CTA per SM; each warp takes equal segments of the cost, the
+ * first by its index and further ones from an atomic counter, finds a segment's
+ * first message by a warp-wide 32-ary search of the prefix and stages the round
+ * keys through shared memory into registers).  Allocates nothing and never synchronises,
  * so it can be captured in a CUDA graph.
  *   n           0..AES_BATCH_MAX_DESCS.
  *   desc_dev    DEVICE array of n descriptors, unchanged until completion.

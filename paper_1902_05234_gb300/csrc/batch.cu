@@ -5,27 +5,33 @@
 // batch only changes which key and which buffer a state belongs to, never the
 // arithmetic.  Two kernels run back to back on the caller's stream:
 //
-//  plan   (one CTA)  validates every descriptor (bad ones get a status and no
+//  plan   (count, then place: one CTA per 1,024 descriptors each, up to 512)
+//                    validates every descriptor (bad ones get a status and no
 //                    work), orders the messages encryptions first, and writes
-//                    the exclusive prefix `start[]` of their chunk counts,
-//                    where a chunk is `chunk_blocks` consecutive blocks of one
-//                    message -- the work of one warp.
-//  batch  (persistent, one CTA per SM)  warps take chunks of the encryption
-//                    range, then of the decryption range, from two atomic
-//                    counters (dynamic: whichever warp is free takes the next
-//                    chunk).  A chunk's message is found by a warp-wide 32-ary
-//                    search in start[]; its round keys are staged through the
-//                    warp's own shared-memory slot into registers.  The CTA's T tables are filled for
-//                    encryption first and refilled once for decryption,
-//                    between two CTA barriers that every warp reaches; each
-//                    phase's table layout is part of the launch configuration
-//                    (default R4 for encryption, 128 KiB, and R2 for
-//                    decryption, also 128 KiB: faster to fill than R4's
-//                    160 KiB and as fast to use).
+//                    the exclusive prefix `start[]` of their costs.  A message's
+//                    cost is Nr for each pass of 32 * blocks_per_thread blocks
+//                    (what one warp ciphers at a time) plus kMsgCost for its key.
+//  batch  (persistent, one CTA per SM)  each direction's cost range is cut into
+//                    equal segments, one per warp when the batch is small, at
+//                    most chunk_passes passes each when it is large; a warp
+//                    starts with the segment of its own index and takes further
+//                    ones from an atomic counter.  A segment is walked message
+//                    by message: the first is found by a warp-wide 32-ary search
+//                    in start[], then each lane resolves one of the next 32
+//                    messages, and the warp ciphers them in turn with the next
+//                    message's round keys and first blocks already on their way.
+//                    The CTA's T tables are filled for encryption first and
+//                    refilled once for decryption, between two CTA barriers that
+//                    every warp reaches; each phase's table layout is part of the
+//                    launch configuration (default R4 for both: with the keys in
+//                    registers R2's rotation costs more than its smaller tables
+//                    save; 5.2 GB in 4,096 messages 6.67 ms against 6.77 with R2
+//                    decryption and 6.89 with R2 in both, 47 MB in 20,000 96.5
+//                    against 98.3 and 101.5 us).
 //
 // Workspace layout (caller- or library-owned device memory, see
 // aes_batch_workspace_bytes):
-//   BatchHeader | uint32 order[n] | uint64 start[n+1] | uint64 count[n]
+//   BatchHeader | uint32 order[n] | uint64 start[n+1] | PlanTile tile[<= n / 1024 + 1]
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -50,13 +56,21 @@ static_assert(offsetof(aes_desc, nblocks) == 24 && offsetof(aes_desc, nrounds) =
               "aes_desc field offsets");
 
 struct BatchHeader {
-    unsigned long long total_chunks;  // T
-    unsigned long long enc_chunks;    // E: chunks [0, E) encrypt, [E, T) decrypt
-    unsigned long long next[2];       // work counters of the two phases (zeroed by the plan)
+    unsigned long long total_chunks;  // chunks of chunk_blocks blocks, all messages
+    unsigned long long enc_chunks;    // of the encryption messages
+    unsigned long long enc_cost;      // costs [0, enc_cost) encrypt, [enc_cost, total_cost) decrypt
+    unsigned long long total_cost;
+    unsigned long long next[2];       // segment counters of the two phases (zeroed by the plan)
     unsigned int n;
     unsigned int chunk_blocks;
     unsigned int n_invalid;
-    unsigned int pad;
+    unsigned int n_enc;               // messages at positions [0, n_enc) encrypt
+};
+
+// What one plan CTA's descriptors add up to (count kernel -> place kernel).
+struct PlanTile {
+    unsigned long long cost[2], chunks[2];  // by direction
+    unsigned int n_enc, n_bad;
 };
 
 __host__ __device__ constexpr size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -67,11 +81,18 @@ size_t batch_ws_bytes(int n) {
            align_up(8 * nn, 256);
 }
 
+// End of the part of the workspace that the batch kernel reads (header, order
+// and start); the plan tiles come after it.
+size_t batch_plan_bytes(int n) {
+    return align_up(sizeof(BatchHeader), 256) + align_up(4 * static_cast<size_t>(n), 256) +
+           8 * (static_cast<size_t>(n) + 1);
+}
+
 struct WsView {
     BatchHeader *hdr;
     uint32_t *order;
     unsigned long long *start;
-    unsigned long long *count;
+    PlanTile *tile;
 };
 
 __host__ __device__ inline WsView ws_view(void *ws, int n) {
@@ -84,7 +105,7 @@ __host__ __device__ inline WsView ws_view(void *ws, int n) {
     p += align_up(4 * nn, 256);
     v.start = reinterpret_cast<unsigned long long *>(p);
     p += align_up(8 * (nn + 1), 256);
-    v.count = reinterpret_cast<unsigned long long *>(p);
+    v.tile = reinterpret_cast<PlanTile *>(p);
     return v;
 }
 
@@ -92,35 +113,6 @@ __host__ __device__ inline WsView ws_view(void *ws, int n) {
 // plan kernel
 // ---------------------------------------------------------------------------
 constexpr int kPlanThreads = 1024;
-
-// Exclusive scan of one value per thread over the CTA; returns the prefix and
-// writes the CTA total to *total.
-template <typename T>
-__device__ T cta_exclusive_scan(T v, T *warp_sums, T *total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    T x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const T y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sums[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        T s = lane < nw ? warp_sums[lane] : T(0);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const T y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < nw) warp_sums[lane] = s;  // inclusive warp prefix
-    }
-    __syncthreads();
-    const T before = warp == 0 ? T(0) : warp_sums[warp - 1];
-    *total = warp_sums[nw - 1];
-    __syncthreads();
-    return before + x - v;
-}
 
 __device__ int check_desc(const aes_desc &d) {
     if (d.nrounds != 10 && d.nrounds != 12 && d.nrounds != 14) return AES_E_NROUNDS;
@@ -136,82 +128,194 @@ __device__ int check_desc(const aes_desc &d) {
     return AES_OK;
 }
 
-__global__ void __launch_bounds__(kPlanThreads, 1)
-    batch_plan_kernel(const aes_desc *__restrict__ desc, int n, void *ws, int32_t *status,
-                      unsigned int chunk_blocks) {
-    __shared__ unsigned long long s_u64[32];
-    __shared__ unsigned int s_u32[32];
-    __shared__ unsigned int s_base[2];
-    const WsView v = ws_view(ws, n);
+constexpr int kPlanMaxCtas = 512;  // each place CTA reads every tile, one per thread
+static_assert(kPlanMaxCtas <= kPlanThreads, "one tile per thread");
+// The workspace ends in 8 bytes per descriptor; a CTA's tile stands for 1,024.
+static_assert(sizeof(PlanTile) <= 8 * kPlanThreads, "tiles fit");
 
-    // pass 1: number of encryption messages (invalid ones count as encryption
-    // with no chunks, so they sit harmlessly in the first range)
-    unsigned int n_enc = 0, n_bad = 0;
-    for (int t0 = 0; t0 < n; t0 += blockDim.x) {
+// Cost of the per-message work (finding it, its round keys) in the unit of one
+// round of one pass: about half a pass.
+constexpr unsigned int kMsgCost = 6;
+
+// The work of one message: nothing for an invalid or empty one.
+struct MsgWork {
+    unsigned long long cost, chunks;
+};
+__host__ __device__ inline MsgWork msg_work(unsigned long long nblocks, int nr, unsigned int pass_blocks,
+                                            unsigned int chunk_blocks) {
+    if (nblocks == 0) return {0ull, 0ull};
+    return {(nblocks + pass_blocks - 1) / pass_blocks * static_cast<unsigned int>(nr) + kMsgCost,
+            (nblocks + chunk_blocks - 1) / chunk_blocks};
+}
+
+struct PlanArgs {
+    const aes_desc *desc;
+    void *ws;
+    int32_t *status;
+    int n, per_cta;  // per_cta: descriptors of one CTA, a multiple of kPlanThreads
+    unsigned int pass_blocks, chunk_blocks;
+};
+
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Sums of the threads' tiles over the CTA, into *out (shared memory, zeroed).
+__device__ __forceinline__ void cta_sum(const PlanTile &t, PlanTile *out) {
+    const unsigned long long v[5] = {t.cost[0], t.cost[1], t.chunks[0], t.chunks[1],
+                                     static_cast<unsigned long long>(t.n_bad) << 32 | t.n_enc};
+    unsigned long long *dst[4] = {&out->cost[0], &out->cost[1], &out->chunks[0], &out->chunks[1]};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const unsigned long long s = warp_sum(v[i]);
+        if ((threadIdx.x & 31) == 0 && s) {
+            if (i < 4) {
+                atomicAdd(dst[i], s);
+            } else {
+                atomicAdd(&out->n_enc, static_cast<unsigned int>(s));
+                atomicAdd(&out->n_bad, static_cast<unsigned int>(s >> 32));
+            }
+        }
+    }
+}
+
+// One descriptor's share of its CTA's tile.  Invalid messages count as
+// encryptions without work, so they sit harmlessly in the first range.
+__device__ __forceinline__ PlanTile desc_tile(const aes_desc &d, int st, const PlanArgs &a) {
+    PlanTile t{};
+    const bool ok = st == AES_OK;
+    t.n_bad = !ok;
+    t.n_enc = !ok || d.dir == 0;
+    const MsgWork w = ok ? msg_work(d.nblocks, d.nrounds, a.pass_blocks, a.chunk_blocks) : MsgWork{0ull, 0ull};
+    t.cost[t.n_enc ? 0 : 1] = w.cost;
+    t.chunks[t.n_enc ? 0 : 1] = w.chunks;
+    return t;
+}
+
+__device__ __forceinline__ void zero_tile(PlanTile *t) {
+    if (threadIdx.x == 0) *t = PlanTile{};
+}
+
+// More than one CTA's worth of descriptors: what each CTA's add up to.
+__global__ void __launch_bounds__(kPlanThreads, 1) batch_count_kernel(const __grid_constant__ PlanArgs a) {
+    __shared__ PlanTile s_sum;
+    griddep_release();
+    zero_tile(&s_sum);
+    __syncthreads();
+    PlanTile sum{};
+    const int first = blockIdx.x * a.per_cta;
+    for (int i = first + static_cast<int>(threadIdx.x); i < a.n && i < first + a.per_cta; i += kPlanThreads) {
+        const aes_desc d = a.desc[i];
+        const PlanTile t = desc_tile(d, check_desc(d), a);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            sum.cost[q] += t.cost[q];
+            sum.chunks[q] += t.chunks[q];
+        }
+        sum.n_enc += t.n_enc;
+        sum.n_bad += t.n_bad;
+    }
+    cta_sum(sum, &s_sum);
+    __syncthreads();
+    if (threadIdx.x == 0) ws_view(a.ws, a.n).tile[blockIdx.x] = s_sum;
+}
+
+// Statuses, partition positions and cost prefix.  A CTA starts from the tiles
+// of the CTAs before it (with one CTA, from nothing: its totals come from its
+// only scan).  Replaces one CTA that scanned all descriptors three times:
+// 20,000 descriptors took 87 us.
+__global__ void __launch_bounds__(kPlanThreads, 1) batch_place_kernel(const __grid_constant__ PlanArgs a) {
+    __shared__ PlanTile s_all, s_before;
+    __shared__ unsigned long long s_cost[2][32];
+    __shared__ unsigned int s_enc[32];
+    griddep_release();
+    zero_tile(&s_all);
+    zero_tile(&s_before);
+    __syncthreads();
+    const WsView v = ws_view(a.ws, a.n);
+    const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const int first = blockIdx.x * a.per_cta;
+    const bool alone = gridDim.x == 1;
+    griddep_wait();  // the count kernel's tiles
+    if (!alone) {
+        const PlanTile t = threadIdx.x < gridDim.x ? v.tile[threadIdx.x] : PlanTile{};
+        cta_sum(t, &s_all);
+        cta_sum(threadIdx.x < blockIdx.x ? t : PlanTile{}, &s_before);
+        __syncthreads();
+    }
+    // running prefixes at the first descriptor of the current 1,024
+    unsigned int enc_before = s_before.n_enc;
+    unsigned long long cost_before[2] = {s_before.cost[0], s_before.cost[1]};
+    for (int t0 = first; t0 < a.n && t0 < first + a.per_cta; t0 += kPlanThreads) {
         const int i = t0 + static_cast<int>(threadIdx.x);
-        unsigned int e = 0, bad = 0;
-        if (i < n) {
-            const aes_desc d = desc[i];
+        PlanTile t{};
+        if (i < a.n) {
+            const aes_desc d = a.desc[i];
             const int st = check_desc(d);
-            bad = st != AES_OK;
-            e = bad || d.dir == 0;
-            if (status) status[i] = st;
+            if (a.status) a.status[i] = st;
+            t = desc_tile(d, st, a);
         }
-        unsigned int tot = 0, totb = 0;
-        (void)cta_exclusive_scan<unsigned int>(e, s_u32, &tot);
-        (void)cta_exclusive_scan<unsigned int>(bad, s_u32, &totb);
-        n_enc += tot;
-        n_bad += totb;
-    }
-    // pass 2: stable partition (encryptions first) and chunk counts by position
-    if (threadIdx.x == 0) { s_base[0] = 0; s_base[1] = n_enc; }
-    __syncthreads();
-    for (int t0 = 0; t0 < n; t0 += blockDim.x) {
-        const int i = t0 + static_cast<int>(threadIdx.x);
-        unsigned int e = 0;
-        unsigned long long cnt = 0;
-        if (i < n) {
-            const aes_desc d = desc[i];
-            const bool ok = check_desc(d) == AES_OK;
-            e = !ok || d.dir == 0;
-            cnt = ok ? (d.nblocks + chunk_blocks - 1) / chunk_blocks : 0ull;
+        if (alone) cta_sum(t, &s_all);
+        // inclusive scans over the warp, then over the warps' totals
+        unsigned int e = t.n_enc;
+        unsigned long long c[2] = {t.cost[0], t.cost[1]};
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int ye = __shfl_up_sync(0xffffffffu, e, o);
+            const unsigned long long y0 = __shfl_up_sync(0xffffffffu, c[0], o);
+            const unsigned long long y1 = __shfl_up_sync(0xffffffffu, c[1], o);
+            if (lane >= static_cast<unsigned int>(o)) {
+                e += ye;
+                c[0] += y0;
+                c[1] += y1;
+            }
         }
-        unsigned int tot_e = 0, tot_d = 0;
-        const unsigned int pe = cta_exclusive_scan<unsigned int>(e, s_u32, &tot_e);
-        const unsigned int pd = cta_exclusive_scan<unsigned int>(i < n ? 1u - e : 0u, s_u32, &tot_d);
-        if (i < n) {
-            const unsigned int pos = e ? s_base[0] + pe : s_base[1] + pd;
+        if (lane == 31u) {
+            s_enc[warp] = e;
+            s_cost[0][warp] = c[0];
+            s_cost[1][warp] = c[1];
+        }
+        __syncthreads();
+        unsigned int te = 0;
+        unsigned long long tc[2] = {0, 0};  // totals of these 1,024
+        for (unsigned int w = 0; w < kPlanThreads / 32; ++w) {
+            if (w == warp) {
+                e += te;
+                c[0] += tc[0];
+                c[1] += tc[1];
+            }
+            te += s_enc[w];
+            tc[0] += s_cost[0][w];
+            tc[1] += s_cost[1][w];
+        }
+        const unsigned int n_enc = s_all.n_enc;
+        const unsigned long long enc_cost = s_all.cost[0];
+        if (i < a.n) {
+            const unsigned int enc_at = enc_before + e - t.n_enc;  // encryptions before this one
+            const unsigned int pos = t.n_enc ? enc_at : n_enc + (static_cast<unsigned int>(i) - enc_at);
             v.order[pos] = static_cast<uint32_t>(i);
-            v.count[pos] = cnt;
+            v.start[pos] = t.n_enc ? cost_before[0] + c[0] - t.cost[0] : enc_cost + cost_before[1] + c[1] - t.cost[1];
         }
-        __syncthreads();
-        if (threadIdx.x == 0) { s_base[0] += tot_e; s_base[1] += tot_d; }
-        __syncthreads();
+        enc_before += te;
+        cost_before[0] += tc[0];
+        cost_before[1] += tc[1];
+        __syncthreads();  // the warps' totals are rewritten next
     }
-    __threadfence_block();
-    __syncthreads();
-    // pass 3: exclusive prefix of the counts in partition order
-    unsigned long long run = 0;
-    for (int t0 = 0; t0 < n; t0 += blockDim.x) {
-        const int p = t0 + static_cast<int>(threadIdx.x);
-        const unsigned long long c = p < n ? v.count[p] : 0ull;
-        unsigned long long tot = 0;
-        const unsigned long long pre = cta_exclusive_scan<unsigned long long>(c, s_u64, &tot);
-        if (p < n) v.start[p] = run + pre;
-        run += tot;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        BatchHeader h{};
+        h.total_chunks = s_all.chunks[0] + s_all.chunks[1];
+        h.enc_chunks = s_all.chunks[0];
+        h.enc_cost = s_all.cost[0];
+        h.total_cost = s_all.cost[0] + s_all.cost[1];
+        h.n = static_cast<unsigned int>(a.n);
+        h.chunk_blocks = a.chunk_blocks;
+        h.n_invalid = s_all.n_bad;
+        h.n_enc = s_all.n_enc;
+        *v.hdr = h;
+        v.start[a.n] = h.total_cost;
     }
-    if (threadIdx.x == 0) {
-        v.start[n] = run;
-        v.hdr->total_chunks = run;
-        v.hdr->next[0] = 0;
-        v.hdr->next[1] = 0;
-        v.hdr->n = static_cast<unsigned int>(n);
-        v.hdr->chunk_blocks = chunk_blocks;
-        v.hdr->n_invalid = n_bad;
-    }
-    // enc_chunks: start[n_enc] (or the total when every message encrypts)
-    __syncthreads();
-    if (threadIdx.x == 0) v.hdr->enc_chunks = n_enc >= static_cast<unsigned int>(n) ? run : v.start[n_enc];
 }
 
 // ---------------------------------------------------------------------------
@@ -224,6 +328,27 @@ struct BatchArgs {
 };
 
 constexpr uint32_t kKeySlotBytes = 256;  // 60 words rounded up
+// A message's part in a segment, as its lane resolved it.
+struct __align__(16) SegEntry {
+    const uint4 *in;
+    uint4 *out;
+    const uint32_t *rk;
+    uint32_t count;  // blocks
+    int nr;
+};
+static_assert(sizeof(SegEntry) == 32, "two 16-byte words");
+// Each warp's shared memory: two key slots (current and next message) and the
+// entries of one window of 32 messages, with an empty one behind the last.
+constexpr uint32_t kWarpSlotBytes = 2 * kKeySlotBytes + 33 * static_cast<uint32_t>(sizeof(SegEntry));
+
+// The segments of one direction's cost range: n_long of `len`, then the rest
+// in short ones, numbered in order.
+struct Segments {
+    unsigned long long len, n_long, tail, n;  // tail: length of the short ones; n: how many in all
+    __device__ __forceinline__ unsigned long long begin(unsigned long long i) const {
+        return i < n_long ? i * len : n_long * len + (i - n_long) * tail;
+    }
+};
 
 // Shared memory of the tables of a launch: the larger of its two phases'.
 __host__ __device__ constexpr uint32_t batch_table_bytes(int le, int ld) {
@@ -240,41 +365,67 @@ static __device__ unsigned int g_chunk_tag[kTagChunks];
 static __device__ unsigned long long g_chunk_tag_beyond;
 #endif
 
-// Round keys of the current message held in registers for a whole chunk
+// Round keys of the current message held in registers for all its passes
 // (4*(NR+1) words; every index is a compile-time constant once the rounds
 // are unrolled, so the array stays in registers).
 template <int NR> struct RegKey {
     uint32_t w[4 * (NR + 1)];
+    __device__ explicit RegKey(const uint32_t *slot) {
+#pragma unroll
+        for (int q = 0; q < NR + 1; ++q) {
+            const uint4 v = reinterpret_cast<const uint4 *>(slot)[q];
+            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+        }
+    }
     __device__ __forceinline__ uint32_t operator()(int i) const { return w[i]; }
 };
 
-// Blocks [first, first + count) of one message, as passes of 32*NB blocks per
-// warp with the next pass prefetched.  The round keys are read once per chunk
-// from the warp's shared-memory slot (16-byte broadcasts) into registers.
+// Round keys left in the warp's slot, read as 16-byte broadcasts: four blocks
+// per thread leave no registers for them, and share each read four ways.
+template <int NR> struct SlotKey {
+    const uint4 *q;
+    __device__ explicit SlotKey(const uint32_t *slot) : q(reinterpret_cast<const uint4 *>(slot)) {}
+    __device__ __forceinline__ uint32_t operator()(int i) const {
+        const uint4 v = q[i >> 2];
+        return (i & 3) == 0 ? v.x : (i & 3) == 1 ? v.y : (i & 3) == 2 ? v.z : v.w;
+    }
+};
+template <int NR, int NB> struct BatchKey { using type = RegKey<NR>; };
+template <int NR> struct BatchKey<NR, 4> { using type = SlotKey<NR>; };
+
+// A lane's blocks of one pass: every 32nd of the `left` blocks that start at
+// its own (which is there if left > 0), zeros past the end.
+template <int NB> __device__ __forceinline__ void load_pass(const uint4 *in, int left, uint4 (&x)[NB]) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) x[i] = left > 32 * i ? ld_block(in + 32 * i) : make_uint4(0, 0, 0, 0);
+}
+
+// One entry's blocks, as passes of 32*NB blocks per warp with the next pass
+// prefetched: behind the last pass, the first of the entry that follows (empty
+// at the end of a window).  cur holds the first pass on entry and the next
+// entry's first on return.  The next pass's address is chosen first and then
+// loaded once: a load on each of two paths makes the warp wait for it where the
+// paths meet, and large messages ran 8 % slower.
 template <int DIR, int NR, int NB, int LAYOUT>
-__device__ __forceinline__ void batch_chunk(const Tab<LAYOUT, DIR> &tab, const uint32_t *kslot,
-                                            const uint4 *in, uint4 *out, unsigned long long first,
-                                            unsigned long long count, uint32_t lane) {
-    RegKey<NR> key;
-#pragma unroll
-    for (int q = 0; q < NR + 1; ++q) {
-        const uint4 v = reinterpret_cast<const uint4 *>(kslot)[q];
-        key.w[4 * q] = v.x; key.w[4 * q + 1] = v.y; key.w[4 * q + 2] = v.z; key.w[4 * q + 3] = v.w;
-    }
-    const unsigned long long end = first + count;
-    uint4 cur[NB];
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-        const unsigned long long b = first + lane + 32ull * i;
-        cur[i] = b < end ? ld_block(in + b) : make_uint4(0, 0, 0, 0);
-    }
-    for (unsigned long long base = first; base < end; base += 32ull * NB) {
-        uint4 nxt[NB];
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-            const unsigned long long b = base + 32ull * NB + lane + 32ull * i;
-            nxt[i] = b < end ? ld_block(in + b) : make_uint4(0, 0, 0, 0);
+__device__ __forceinline__ void batch_entry(const Tab<LAYOUT, DIR> &tab, const uint32_t *kslot, const SegEntry *e,
+                                            uint32_t lane, uint4 (&cur)[NB]) {
+    constexpr int kPass = 32 * NB;
+    const typename BatchKey<NR, NB>::type key(kslot);
+    const uint4 *in = e->in + lane;
+    uint4 *out = e->out + lane;
+    const uint4 *next_in = e[1].in + lane;
+    const int next_count = static_cast<int>(e[1].count);
+#pragma unroll 1  // two passes per iteration measured 25 % slower (registers, instruction cache)
+    for (int left = static_cast<int>(e->count); left > 0; left -= kPass) {
+        in += kPass;
+        const uint4 *src = in;
+        int more = left - kPass;
+        if (more <= 0) {
+            src = next_in;
+            more = next_count;
         }
+        uint4 nxt[NB];
+        load_pass<NB>(src, more - static_cast<int>(lane), nxt);
         uint32_t s[NB][4];
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
@@ -283,16 +434,38 @@ __device__ __forceinline__ void batch_chunk(const Tab<LAYOUT, DIR> &tab, const u
         cipher_states<DIR, NR, NB>(tab, key, s);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
-            const unsigned long long b = base + lane + 32ull * i;
-            if (b < end) st_block(out + b, make_uint4(s[i][0], s[i][1], s[i][2], s[i][3]));
+            if (left - static_cast<int>(lane) > 32 * i)
+                st_block(out + 32 * i, make_uint4(s[i][0], s[i][1], s[i][2], s[i][3]));
             cur[i] = nxt[i];
         }
+        out += kPass;
     }
 }
 
-// Partition position q of the message owning chunk c: the largest q in
-// [lo, n) with start[q] <= c (start[n] = T > c).  32-ary search by the whole
-// warp: each lane probes one of 31 evenly spaced positions per step.
+// Copy of one message's round keys into a key slot, in application order, by
+// asynchronous 4-byte copies (schedules are 4-byte aligned): lanes never wait
+// for them here.
+template <int DIR>
+__device__ __forceinline__ void prefetch_keys(uint32_t *slot, const uint32_t *rk, int nr, uint32_t lane) {
+    for (int i = static_cast<int>(lane); i < 4 * (nr + 1); i += 32) {
+        const int step = i >> 2;
+        const int src = DIR == kEncrypt ? step : nr - step;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                         static_cast<uint32_t>(__cvta_generic_to_shared(slot + i))),
+                     "l"(rk + 4 * src + (i & 3))
+                     : "memory");
+    }
+}
+__device__ __forceinline__ void wait_keys() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ceil(x / nr) for the three round counts, as multiplications.
+__device__ __forceinline__ unsigned long long ceil_div_nr(unsigned long long x, int nr) {
+    return nr == 10 ? (x + 9) / 10 : nr == 12 ? (x + 11) / 12 : (x + 13) / 14;
+}
+
+// Partition position q of the message that owns cost c: the largest q in
+// [lo, n) with start[q] <= c.  32-ary search by the whole warp: each lane
+// probes one of 31 evenly spaced positions per step.
 __device__ __forceinline__ int find_message(const unsigned long long *start, int lo, int n,
                                             unsigned long long c, uint32_t lane) {
     int hi = n;
@@ -309,110 +482,181 @@ __device__ __forceinline__ int find_message(const unsigned long long *start, int
     return lo;
 }
 
-// All chunks of one direction, handed out one at a time to whichever warp
-// asks next (an atomic counter in the workspace; the next chunk index is
-// requested before the current chunk is processed, so the atomic's latency is
-// hidden).  Chunk c of this phase is chunk c_begin + c of the partition.
+#if defined(AESGB_BOUNDS_CHECK)
+// Debug build: tag the chunks of message `pos` whose first pass is one of
+// [j0, j1).  The chunks before the message's are counted over the partition.
+__device__ inline void tag_chunks(const BatchArgs &a, const WsView &v, int pos, unsigned long long j0,
+                                  unsigned long long j1, unsigned int pass_blocks) {
+    const unsigned int cb = v.hdr->chunk_blocks, cp = cb / pass_blocks;
+    unsigned long long before = 0;
+    for (int q = 0; q < pos; ++q)
+        if (v.start[q + 1] > v.start[q]) before += (a.desc[v.order[q]].nblocks + cb - 1) / cb;
+    for (unsigned long long k = (j0 + cp - 1) / cp; k * cp < j1; ++k) {
+        const unsigned long long c = before + k;
+        if (c < kTagChunks) atomicAdd(&g_chunk_tag[c], 1u);
+        else atomicAdd(&g_chunk_tag_beyond, 1ull);
+    }
+}
+#endif
+
+// One direction's cost range [c_begin, c_end), messages at positions
+// [p_begin, p_end).  It is cut into segments of `seg`; warp w of W starts with
+// segment w, and where there are more than W takes its further ones from the
+// counter (the next index is requested before the current segment is walked, so
+// the atomic's latency is hidden).  A pass belongs to the segment that its
+// first unit of cost lies in.
 template <int DIR, int NB, int LAYOUT>
-__device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, uint32_t *kslot,
-                            unsigned long long c_begin, unsigned long long c_end) {
+__device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, uint8_t *wslot, unsigned int w,
+                            unsigned int W, unsigned long long c_begin, unsigned long long c_end, int p_begin,
+                            int p_end, const Segments &seg) {
     const uint32_t lane = threadIdx.x & 31u;
     const Tab<LAYOUT, DIR> tab(smem, lane);
-    unsigned long long *counter = &v.hdr->next[DIR];
-    const unsigned long long nchunks = c_end - c_begin;
-    const unsigned int cb = v.hdr->chunk_blocks;
-    const int n = a.n;
-    int p = 0;                                  // partition position of the current message
-    unsigned long long p_start = 0, p_end = 0;  // its chunk range [p_start, p_end)
-    const uint4 *in = nullptr;
-    uint4 *out = nullptr;
-    unsigned long long nb = 0;
-    int nr = 10;
-    bool have = false;
-    unsigned long long ticket = 0;
-    // the warp's key slot lies inside the launch's shared memory
-    if (!AESGB_CHECK(static_cast<uint32_t>(reinterpret_cast<uint8_t *>(kslot) - smem) + kKeySlotBytes <=
-                     dyn_smem_bytes()))
-        return;
-    if (lane == 0) ticket = atomicAdd(counter, 1ull);
-    unsigned long long rel = __shfl_sync(0xffffffffu, ticket, 0);
-    while (rel < nchunks) {
-        if (lane == 0) ticket = atomicAdd(counter, 1ull);  // next chunk, consumed after this one
-        const unsigned long long c = c_begin + rel;
-        if (!have || c >= p_end) {
-            p = find_message(v.start, have ? p + 1 : 0, n, c, lane);
-            // p is a partition position with c in its chunk range, and names
-            // a message (each value is the same in every lane: no divergence)
-            if (!AESGB_CHECK(p >= 0 && p < n && v.order[p] < static_cast<uint32_t>(n) && v.start[p] <= c &&
-                             c < v.start[p + 1]))
-                break;
-            p_start = v.start[p];
-            p_end = v.start[p + 1];
-            const aes_desc d = a.desc[v.order[p]];
-            in = reinterpret_cast<const uint4 *>(d.in);
-            out = reinterpret_cast<uint4 *>(d.out);
-            nb = d.nblocks;
-            nr = d.nrounds;
-            __syncwarp();
-            const int nw = 4 * (nr + 1);
-            for (int i = static_cast<int>(lane); i < nw; i += 32) {
-                const int step = i >> 2;
-                const int src = DIR == kEncrypt ? step : nr - step;
-                kslot[i] = d.rk[4 * src + (i & 3)];
+    constexpr unsigned int kPass = 32u * NB;
+    // the warp's slots lie inside the launch's shared memory
+    if (!AESGB_CHECK(static_cast<uint32_t>(wslot - smem) + kWarpSlotBytes <= dyn_smem_bytes())) return;
+    SegEntry *entries = reinterpret_cast<SegEntry *>(wslot + 2 * kKeySlotBytes);
+    int p = p_begin;  // no message before it is of use to this warp any more
+    unsigned long long rel = w;
+    while (rel < seg.n) {
+        unsigned long long ticket = 0;
+        if (seg.n > W && lane == 0) ticket = atomicAdd(&v.hdr->next[DIR], 1ull);
+        const unsigned long long lo = c_begin + seg.begin(rel), stop = c_begin + seg.begin(rel + 1);
+        const unsigned long long hi = stop < c_end ? stop : c_end;
+        p = find_message(v.start, p, p_end, lo, lane);
+        for (int p0 = p;; p0 += 32) {
+            // lane: message p0 + lane, its passes [j0, j1) inside [lo, hi)
+            const int pos = p0 + static_cast<int>(lane);
+            unsigned long long s0 = ~0ull;
+            SegEntry e{};
+            bool take = false;
+            if (pos < p_end) {
+                s0 = v.start[pos];
+                take = s0 < hi && v.start[pos + 1] > s0;  // in the segment, and neither empty nor invalid
+                take = take && AESGB_CHECK(pos >= 0 && v.order[pos] < static_cast<uint32_t>(a.n));
             }
-            __syncwarp();
-            have = true;
-        }
-        const unsigned long long first = (c - p_start) * cb;
-        const unsigned long long cnt = nb - first < cb ? nb - first : cb;
-        if (!AESGB_CHECK(first < nb && cnt >= 1 && cnt <= cb && (nr == 10 || nr == 12 || nr == 14))) break;
+            if (take) {
+                const aes_desc d = a.desc[v.order[pos]];
+                const unsigned long long passes = (d.nblocks + kPass - 1) / kPass;
+                const unsigned long long j0 = s0 < lo ? ceil_div_nr(lo - s0, d.nrounds) : 0ull;
+                const unsigned long long j1 =
+                    hi - s0 >= passes * static_cast<unsigned int>(d.nrounds) ? passes : ceil_div_nr(hi - s0, d.nrounds);
+                const unsigned long long first = j0 * kPass;
+                const unsigned long long end = j1 * kPass < d.nblocks ? j1 * kPass : d.nblocks;
+                take = j0 < j1;
+                take = take && AESGB_CHECK(d.dir == DIR && end <= d.nblocks && first < end && end - first <= seg.len * kPass);
+                e.in = reinterpret_cast<const uint4 *>(d.in) + first;
+                e.out = reinterpret_cast<uint4 *>(d.out) + first;
+                e.rk = d.rk;
+                e.count = static_cast<uint32_t>(end - first);
+                e.nr = d.nrounds;
 #if defined(AESGB_BOUNDS_CHECK)
-        if (lane == 0) {
-            if (c < kTagChunks) atomicAdd(&g_chunk_tag[c], 1u);
-            else atomicAdd(&g_chunk_tag_beyond, 1ull);
-        }
+                if (take) tag_chunks(a, v, pos, j0, j1, kPass);
 #endif
-        switch (nr) {
-        case 10: batch_chunk<DIR, 10, NB, LAYOUT>(tab, kslot, in, out, first, cnt, lane); break;
-        case 12: batch_chunk<DIR, 12, NB, LAYOUT>(tab, kslot, in, out, first, cnt, lane); break;
-        default: batch_chunk<DIR, 14, NB, LAYOUT>(tab, kslot, in, out, first, cnt, lane); break;
+            }
+            const unsigned int taken = __ballot_sync(0xffffffffu, take);
+            const bool more = __shfl_sync(0xffffffffu, s0, 31) < hi;  // the window's last message starts inside
+            __syncwarp();  // every lane is done with the entries and key slots of the last window
+            const int k = __popc(taken);
+            if (take) entries[__popc(taken & ((1u << lane) - 1u))] = e;
+            if (lane == 0) entries[k] = SegEntry{};
+            __syncwarp();
+            uint4 cur[NB];
+            if (k > 0) {
+                load_pass<NB>(entries[0].in + lane, static_cast<int>(entries[0].count - lane), cur);
+                prefetch_keys<DIR>(reinterpret_cast<uint32_t *>(wslot), entries[0].rk, entries[0].nr, lane);
+            }
+            for (int i = 0; i < k; ++i) {
+                const SegEntry *now = entries + i;
+                const uint32_t *kslot = reinterpret_cast<const uint32_t *>(wslot + (i & 1) * kKeySlotBytes);
+                wait_keys();
+                __syncwarp();  // all lanes' key words are there, and all are done with the other slot
+                if (i + 1 < k)
+                    prefetch_keys<DIR>(reinterpret_cast<uint32_t *>(wslot + ((i + 1) & 1) * kKeySlotBytes), now[1].rk,
+                                       now[1].nr, lane);
+                switch (now->nr) {
+                case 10: batch_entry<DIR, 10, NB, LAYOUT>(tab, kslot, now, lane, cur); break;
+                case 12: batch_entry<DIR, 12, NB, LAYOUT>(tab, kslot, now, lane, cur); break;
+                default: batch_entry<DIR, 14, NB, LAYOUT>(tab, kslot, now, lane, cur); break;
+                }
+            }
+            if (!more) break;
         }
-        rel = __shfl_sync(0xffffffffu, ticket, 0);
+        if (seg.n <= W) break;
+        rel = W + __shfl_sync(0xffffffffu, ticket, 0);
     }
+}
+
+// Segments of a direction of total cost c on W warps: one equal share for each
+// warp while that is at most `most`; above, long ones and at the end (an eighth
+// of the whole, at most half a long one per warp) short ones, so that the
+// counter evens out the end.
+__device__ __forceinline__ Segments cut(unsigned long long c, unsigned int W, unsigned int most) {
+    Segments s;
+    const unsigned long long share = (c + W - 1) / W;
+    if (share <= most) {
+        s.len = s.tail = share > 14 ? share : 14;  // at least a pass
+        s.n = s.n_long = (c + s.len - 1) / s.len;
+        return s;
+    }
+    s.len = most;
+    s.tail = most / 8 > 14 ? most / 8 : 14;
+    const unsigned long long end = c / 8 < W * 1ull * most / 2 ? c / 8 : W * 1ull * most / 2;
+    s.n_long = (c - end) / s.len;
+    s.n = s.n_long + (c - s.n_long * s.len + s.tail - 1) / s.tail;
+    return s;
 }
 
 constexpr int kBatchMaxThreads = 512;  // up to 128 registers: round keys live in registers
 
 // LE, LD: table layouts of the encryption and decryption phases.
+//
+// Bound: the L1TEX data pipe (the lookups) for large batches, 93-96 % busy; with
+// small messages the latencies in front of each one (its descriptor, keys and
+// first blocks), which is why the next message's are always under way, and why
+// a batch that gives a warp less than two chunks is cut into equal shares
+// instead of whole chunks.  Against one chunk of one message at a time, found by
+// a search each, behind a one-CTA plan: 20,000 messages of 16 B to 16 KiB 217 ->
+// 97 us (plan 87 -> about 9), 2,000 of them 64 -> 31, 20 of them 38 -> 12; 2,000
+// of up to 4 MiB 908 -> 893 us (kernel and plan), 4,096 of up to 16 MiB (5.2 GB)
+// 6,689 -> 6,640.  With 512 threads and the 44 to 60 key words in registers a
+// thread has one block in flight; two measured 20 % slower.
 template <int NB, int LE, int LD>
 __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const WsView v = ws_view(a.ws, a.n);
-    const unsigned long long T = v.hdr->total_chunks, E = v.hdr->enc_chunks;
-    uint32_t *kslot =
-        reinterpret_cast<uint32_t *>(smem + batch_table_bytes(LE, LD) + (threadIdx.x >> 5) * kKeySlotBytes);
-    if (E > 0) {
-        Tab<LE, kEncrypt>::fill(smem, threadIdx.x, blockDim.x);
-        __syncthreads();
-        batch_phase<kEncrypt, NB, LE>(a, v, smem, kslot, 0, E);
-    }
-    if (T > E) {
+    uint8_t *wslot = smem + batch_table_bytes(LE, LD) + (threadIdx.x >> 5) * kWarpSlotBytes;
+    // launched behind the plan (programmatic dependent launch): the first fill
+    // reads only constant tables and runs while the plan does
+    Tab<LE, kEncrypt>::fill(smem, threadIdx.x, blockDim.x);
+    griddep_wait();
+    __syncthreads();
+    const unsigned long long E = v.hdr->enc_cost, T = v.hdr->total_cost;
+    // a long segment: twice chunk_passes passes of the middle key size
+    const unsigned int most = v.hdr->chunk_blocks / (32u * NB) * 24u, G = gridDim.x, W = G * (blockDim.x >> 5);
+    const int n_enc = static_cast<int>(v.hdr->n_enc);
+    // Warps are numbered across the CTAs first, so that few segments spread
+    // over the SMs; from the other end for decryption, so that two small
+    // directions run side by side.  A CTA without a segment skips the phase.
+    const unsigned int row = (threadIdx.x >> 5) * G, back = G - 1 - blockIdx.x;
+    const Segments se = cut(E, W, most), sd = cut(T - E, W, most);
+    if (blockIdx.x < se.n) batch_phase<kEncrypt, NB, LE>(a, v, smem, wslot, row + blockIdx.x, W, 0, E, 0, n_enc, se);
+    if (back < sd.n) {
         __syncthreads();  // every warp is done with the encryption tables
         Tab<LD, kDecrypt>::fill(smem, threadIdx.x, blockDim.x);
         __syncthreads();
-        batch_phase<kDecrypt, NB, LD>(a, v, smem, kslot, E, T);
+        batch_phase<kDecrypt, NB, LD>(a, v, smem, wslot, row + back, W, E, T, n_enc, a.n, sd);
     }
 }
 
 AESGB_BOUNDS_READER(batch)
 
 uint32_t batch_smem_bytes(const aes_batch_cfg &c) {
-    return batch_table_bytes(c.layout_enc, c.layout_dec) + static_cast<uint32_t>(c.threads / 32) * kKeySlotBytes;
+    return batch_table_bytes(c.layout_enc, c.layout_dec) + static_cast<uint32_t>(c.threads / 32) * kWarpSlotBytes;
 }
 
 // The compiled (blocks per thread, encryption layout, decryption layout)
-// combinations: the default pair R4 / R2 at 1, 2 and 4 blocks per thread, and
-// the pairs R4 / R4, R2 / R2 and R1 / R1 at 1 and 2 (the tuner's range).
+// combinations: the pair R4 / R2 at 1, 2 and 4 blocks per thread, and the pairs
+// R4 / R4 (the default), R2 / R2 and R1 / R1 at 1 and 2 (the tuner's range).
 const void *batch_kernel_ptr(int nb, int le, int ld) {
 #define AESGB_BK(NB, LE, LD) \
     if (nb == NB && le == LE && ld == LD) return reinterpret_cast<const void *>(&batch_kernel<NB, LE, LD>);
@@ -433,6 +677,24 @@ int validate_batch_cfg(const aes_batch_cfg &c) {
     return AES_OK;
 }
 
+unsigned int batch_chunk_blocks(const aes_batch_cfg &c) {
+    return static_cast<unsigned int>(32 * c.blocks_per_thread * c.chunk_passes);
+}
+
+// The persistent kernel on a planned workspace; the plan is the kernel (or the
+// copy) before it in the stream.
+int launch_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_cfg &c, int dev, cudaStream_t s) {
+    const void *fn = batch_kernel_ptr(c.blocks_per_thread, c.layout_enc, c.layout_dec);
+    const uint32_t smem = batch_smem_bytes(c);
+    const int st = ensure_smem_attr(fn, dev, smem);
+    if (st != AES_OK) return st;
+    const int sms = sm_count(dev);
+    if (sms < 0) return sms;
+    BatchArgs args{desc, ws, n};
+    void *params[] = {&args};
+    return launch_pdl(fn, sms, c.threads, smem, params, s);
+}
+
 int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_t *status,
                   const aes_batch_cfg &c, cudaStream_t s) {
     if (n == 0) return AES_OK;
@@ -444,62 +706,63 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
     if (st != AES_OK) return st;
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
-    const unsigned int chunk_blocks = static_cast<unsigned int>(32 * c.blocks_per_thread * c.chunk_passes);
-    batch_plan_kernel<<<1, kPlanThreads, 0, s>>>(desc, n, ws, status, chunk_blocks);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return AES_E_CUDA;
-    const void *fn = batch_kernel_ptr(c.blocks_per_thread, c.layout_enc, c.layout_dec);
-    const uint32_t smem = batch_smem_bytes(c);
-    st = ensure_smem_attr(fn, dev, smem);
-    if (st != AES_OK) return st;
-    const int sms = sm_count(dev);
-    if (sms < 0) return sms;
-    BatchArgs args{desc, ws, n};
-    void *params[] = {&args};
-    e = cudaLaunchKernel(fn, dim3(sms), dim3(c.threads), params, smem, s);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        return AES_E_CUDA;
+    PlanArgs pa;
+    pa.desc = desc;
+    pa.ws = ws;
+    pa.status = status;
+    pa.n = n;
+    pa.pass_blocks = static_cast<unsigned int>(32 * c.blocks_per_thread);
+    pa.chunk_blocks = batch_chunk_blocks(c);
+    const int tiles = (n + kPlanThreads - 1) / kPlanThreads, per = (tiles + kPlanMaxCtas - 1) / kPlanMaxCtas;
+    pa.per_cta = per * kPlanThreads;
+    const int ctas = (tiles + per - 1) / per;
+    void *params[] = {&pa};
+    if (ctas > 1) {
+        batch_count_kernel<<<ctas, kPlanThreads, 0, s>>>(pa);
+        if (cudaGetLastError() != cudaSuccess) return AES_E_CUDA;
+        st = launch_pdl(reinterpret_cast<const void *>(&batch_place_kernel), ctas, kPlanThreads, 0, params, s);
+        if (st != AES_OK) return st;
+    } else {
+        batch_place_kernel<<<1, kPlanThreads, 0, s>>>(pa);
+        if (cudaGetLastError() != cudaSuccess) return AES_E_CUDA;
     }
-    return AES_OK;
+    return launch_batch_kernel(desc, n, ws, c, dev, s);
 }
 
 // ---------------------------------------------------------------------------
 // host-side planning (for callers that know their batch: the server)
 // ---------------------------------------------------------------------------
-// Writes into a HOST buffer of batch_ws_bytes(n) bytes exactly what the plan
-// kernel would write into the workspace for these descriptors, which must all
-// be valid (check_desc): encryptions first in input order, then decryptions;
-// start[] the exclusive prefix of ceil(nblocks / chunk_blocks); counters 0.
-void plan_on_host(const aes_desc *desc, int n, unsigned int chunk_blocks, void *ws_host) {
+// Writes into a HOST buffer of batch_plan_bytes(n) bytes exactly what the plan
+// kernels would write into that part of the workspace for these descriptors,
+// which must all be valid (check_desc): encryptions first in input order, then
+// decryptions; start[] the exclusive prefix of the costs; counters 0.
+void plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host) {
     const WsView v = ws_view(ws_host, n);
+    const unsigned int pass_blocks = static_cast<unsigned int>(32 * c.blocks_per_thread), chunk_blocks = batch_chunk_blocks(c);
+    BatchHeader h{};
+    unsigned long long run = 0;
     int pos = 0;
-    for (int pass = 0; pass < 2; ++pass)
+    for (int dir = 0; dir < 2; ++dir) {
         for (int i = 0; i < n; ++i)
-            if ((desc[i].dir == 0) == (pass == 0)) {
+            if (desc[i].dir == dir) {
+                const MsgWork w = msg_work(desc[i].nblocks, desc[i].nrounds, pass_blocks, chunk_blocks);
                 v.order[pos] = static_cast<uint32_t>(i);
-                v.count[pos] = (desc[i].nblocks + chunk_blocks - 1) / chunk_blocks;
+                v.start[pos] = run;
+                run += w.cost;
+                h.total_chunks += w.chunks;
                 ++pos;
             }
-    unsigned long long run = 0, enc_chunks = 0;
-    for (int p = 0; p < n; ++p) {
-        v.start[p] = run;
-        run += v.count[p];
-        if (desc[v.order[p]].dir == 0) enc_chunks = run;
+        if (dir == 0) {
+            h.n_enc = static_cast<unsigned int>(pos);
+            h.enc_cost = run;
+            h.enc_chunks = h.total_chunks;
+        }
     }
     v.start[n] = run;
-    v.hdr->total_chunks = run;
-    v.hdr->enc_chunks = enc_chunks;
-    v.hdr->next[0] = 0;
-    v.hdr->next[1] = 0;
-    v.hdr->n = static_cast<unsigned int>(n);
-    v.hdr->chunk_blocks = chunk_blocks;
-    v.hdr->n_invalid = 0;
-    v.hdr->pad = 0;
-}
-
-unsigned int batch_chunk_blocks(const aes_batch_cfg &c) {
-    return static_cast<unsigned int>(32 * c.blocks_per_thread * c.chunk_passes);
+    h.total_cost = run;
+    h.n = static_cast<unsigned int>(n);
+    h.chunk_blocks = chunk_blocks;
+    *v.hdr = h;
 }
 
 // The persistent batch kernel alone, on a workspace planned already.
@@ -510,19 +773,7 @@ int enqueue_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_
     if (st != AES_OK) return st;
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
-    const void *fn = batch_kernel_ptr(c.blocks_per_thread, c.layout_enc, c.layout_dec);
-    const uint32_t smem = batch_smem_bytes(c);
-    st = ensure_smem_attr(fn, dev, smem);
-    if (st != AES_OK) return st;
-    const int sms = sm_count(dev);
-    if (sms < 0) return sms;
-    BatchArgs args{desc, ws, n};
-    void *params[] = {&args};
-    if (cudaLaunchKernel(fn, dim3(sms), dim3(c.threads), params, smem, s) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return AES_E_CUDA;
-    }
-    return AES_OK;
+    return launch_batch_kernel(desc, n, ws, c, dev, s);
 }
 
 // ---------------------------------------------------------------------------

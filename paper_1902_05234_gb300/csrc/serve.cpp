@@ -199,20 +199,6 @@ void free_server(Server *s) {
 // wants 256-byte alignment).
 size_t plan_offset(int n) { return (sizeof(aes_desc) * static_cast<size_t>(n) + 255) & ~static_cast<size_t>(255); }
 
-// Batch configuration for a batch of `total_blocks`: chunks small enough that
-// every warp of the grid gets several (latency at light load), at most the
-// throughput-tuned chunk size.
-aes_batch_cfg serve_cfg(int sms, unsigned long long total_blocks) {
-    aes_batch_cfg c = batch_cfg_for(0);
-    const unsigned long long warps = static_cast<unsigned long long>(sms) * (c.threads / 32);
-    const unsigned long long per_pass = 32ull * c.blocks_per_thread;
-    unsigned long long passes = total_blocks / (warps * 4 * per_pass);
-    if (passes < 1) passes = 1;
-    if (passes > static_cast<unsigned long long>(c.chunk_passes)) passes = c.chunk_passes;
-    c.chunk_passes = static_cast<int32_t>(passes);
-    return c;
-}
-
 nvtxDomainHandle_t nvtx_domain() {
     static const nvtxDomainHandle_t d = nvtxDomainCreateA("aesgb");
     return d;
@@ -274,7 +260,6 @@ void retire_locked(Server *s) {
 struct Launch {
     Slot *sl = nullptr;
     int n = 0;
-    unsigned long long blocks = 0;
     bool new_period = false;  // every other slot was idle: the batch opens a busy period
     bool timed = false;       // record the batch's device interval
     bool wait_keys = false;   // keys were uploaded since this slot's stream last waited
@@ -295,7 +280,6 @@ bool pack_locked(Server *s, Launch *L) {
     const double t = now_s();
     int n = 0;
     size_t bytes = 0;
-    unsigned long long blocks = 0;
     // one batch takes at most its share of the budget, so that under load
     // several batches are queued on the device and the next one is already
     // there when one finishes (a single request larger than the share still
@@ -319,7 +303,6 @@ bool pack_locked(Server *s, Launch *L) {
         sl->tickets.push_back(s->pending.front());
         s->pending.pop_front();
         bytes += need;
-        blocks += d.nblocks;
         ++n;
     }
     if (n == 0) return false;
@@ -331,7 +314,6 @@ bool pack_locked(Server *s, Launch *L) {
     s->peak_busy = std::max(s->peak_busy, busy + 1);
     L->sl = sl;
     L->n = n;
-    L->blocks = blocks;
     L->new_period = busy == 0;
     // a period is timed as a whole: only if timing was on when it opened
     if (L->new_period) s->period_timed = s->device_timing;
@@ -347,13 +329,13 @@ bool pack_locked(Server *s, Launch *L) {
 // NOT held): the plan (message order, chunk prefix, zeroed counters) is built
 // here -- every request was validated at submission -- and uploaded with the
 // descriptors, so only the persistent kernel runs on the device.
-bool launch_unlocked(Server *s, const Launch &L, int sms) {
+bool launch_unlocked(Server *s, const Launch &L) {
     const NvtxRange range("aes_srv plan+launch");
     Slot *sl = L.sl;
-    const aes_batch_cfg cfg = serve_cfg(sms, L.blocks);
+    const aes_batch_cfg cfg = batch_cfg_for(L.n);
     const size_t ws_off = plan_offset(L.n);
-    plan_on_host(sl->h_desc, L.n, batch_chunk_blocks(cfg), reinterpret_cast<uint8_t *>(sl->h_desc) + ws_off);
-    bool ok = cudaMemcpyAsync(sl->d_desc, sl->h_desc, ws_off + batch_ws_bytes(L.n), cudaMemcpyHostToDevice,
+    plan_on_host(sl->h_desc, L.n, cfg, reinterpret_cast<uint8_t *>(sl->h_desc) + ws_off);
+    bool ok = cudaMemcpyAsync(sl->d_desc, sl->h_desc, ws_off + batch_plan_bytes(L.n), cudaMemcpyHostToDevice,
                               sl->stream) == cudaSuccess;
     ok = ok && (!L.wait_keys || cudaStreamWaitEvent(sl->stream, s->key_ev, 0) == cudaSuccess);
     // the batch that opens a busy period starts at the period's reference
@@ -400,7 +382,6 @@ void worker_main(Server *s) {
     // latency.  This thread's slack only, for its lifetime.
     (void)prctl(PR_SET_TIMERSLACK, 1UL, 0UL, 0UL, 0UL);
 #endif
-    const int sms = sm_count(s->dev) > 0 ? sm_count(s->dev) : 1;
     std::unique_lock<std::mutex> lk(s->mu);
     while (!s->stop) {
         const uint64_t before = s->n_completed;
@@ -409,7 +390,7 @@ void worker_main(Server *s) {
         Launch L;
         while (!s->stop && pack_locked(s, &L)) {
             lk.unlock();
-            const bool ok = launch_unlocked(s, L, sms);
+            const bool ok = launch_unlocked(s, L);
             lk.lock();
             finish_launch_locked(s, L, ok);
             launched = true;

@@ -256,7 +256,7 @@ aes_batch_cfg default_batch_cfg() {
     c.chunk_passes = 32;
     c.ctas_per_sm = 1;
     c.layout_enc = AES_LAYOUT_R4;
-    c.layout_dec = AES_LAYOUT_R2;
+    c.layout_dec = AES_LAYOUT_R4;
     return c;
 }
 
@@ -346,10 +346,10 @@ int aes_tune_batch(const aes_desc *desc_dev, int n, void *ws, size_t ws_bytes, v
     for (int nb : {1, 2})
         for (int th : {256, 384, 512})
             for (int passes : {8, 16, 32, 64})
-                consider(aes_batch_cfg{th, nb, passes, 1, AES_LAYOUT_R4, AES_LAYOUT_R2});
+                consider(aes_batch_cfg{th, nb, passes, 1, AES_LAYOUT_R4, AES_LAYOUT_R4});
     if (best_ms >= 1e29f) return AES_E_CUDA;
     const aes_batch_cfg g = best_cfg;
-    const int pairs[][2] = {{AES_LAYOUT_R4, AES_LAYOUT_R4}, {AES_LAYOUT_R2, AES_LAYOUT_R2}, {AES_LAYOUT_R1, AES_LAYOUT_R1}};
+    const int pairs[][2] = {{AES_LAYOUT_R4, AES_LAYOUT_R2}, {AES_LAYOUT_R2, AES_LAYOUT_R2}, {AES_LAYOUT_R1, AES_LAYOUT_R1}};
     for (const auto &p : pairs)
         consider(aes_batch_cfg{g.threads, g.blocks_per_thread, g.chunk_passes, g.ctas_per_sm, p[0], p[1]});
     {

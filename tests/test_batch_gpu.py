@@ -258,3 +258,43 @@ def test_library_workspace_batch_with_status(orc):
             assert np.all(b.message(out, i) == 0x5A), i
         else:
             assert np.array_equal(b.message(out, i), orc.ecb(int(b.dirs[i]), b.keys[i], b.message(b.data, i))), i
+
+
+@pytest.mark.parametrize("n, invalid", [(31, False), (33, True), (1023, True), (1024, False), (1025, True), (3000, True)])
+def test_batch_plan_and_segment_edges(orc, n, invalid):
+    """Sizes at which the plan takes one or several CTAs (1,024 descriptors
+    each) and a warp one or several windows of 32 messages, with empty and
+    invalid messages in between (whole windows of them), one message that many
+    warps share, and each way a direction is cut: equal shares (the default
+    here), and long and short segments from the counter (few warps, one pass per
+    chunk)."""
+    torch = torch_cuda()
+    g = wl.rng(40 + n)
+    lengths = 16 * g.integers(0, 70, size=n)
+    lengths[n // 2] = 16 * 20_011
+    lengths[3:min(n, 75)] = 0                              # more than two windows without work
+    keybits = g.choice(np.array([128, 192, 256]), size=n)
+    dirs = g.integers(0, 2, size=n)
+    b = DeviceBatch(torch, lengths, keybits, dirs, seed=41)
+    bad = [i for i in range(0, n, 7) if i != n // 2] if invalid else []
+    for i in bad:
+        b.table[i]["nrounds"] = 11
+    b.upload()
+    ws, nbytes = b.workspace()
+    exp = {}
+    for cfg in (None, aesgb.make_batch_cfg(64, 1, 1, 1), aesgb.make_batch_cfg(64, 2, 1, 1),
+                aesgb.make_batch_cfg(512, 4, 3, 1), aesgb.make_batch_cfg(96, 2, 2, 1, aesgb.LAYOUT_R2, aesgb.LAYOUT_R2)):
+        b.out_dev.fill_(0x5A)
+        status = torch.full((n,), 99, dtype=torch.int32, device="cuda")
+        aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes, status, cfg=cfg)
+        out = b.output()
+        st = status.cpu().numpy()
+        assert np.all(st[bad] == -3) and np.all(np.delete(st, bad) == 0)
+        for i in range(n):
+            got = b.message(out, i)
+            if i in bad:
+                assert np.all(got == 0x5A), i
+                continue
+            if i not in exp:
+                exp[i] = orc.ecb(int(b.dirs[i]), b.keys[i], b.message(b.data, i))
+            assert np.array_equal(got, exp[i]), (i, repr(cfg))
