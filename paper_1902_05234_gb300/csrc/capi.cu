@@ -103,25 +103,30 @@ int validate_cfg(const aes_launch_cfg &c) {
 }
 
 // Grid of a persistent launch: as many CTAs as fit (or as requested), never
-// more than the work needs.
+// more than the work needs.  The first call of a (kernel, device, threads,
+// shared bytes) sets the kernel's shared-memory limit and queries its occupancy;
+// later ones find both behind one lock.
 int persistent_grid(const void *fn, int dev, const aes_launch_cfg &c, uint32_t smem,
                     unsigned long long work_items_per_cta, unsigned long long total_items,
                     int *grid) {
     const int sms = sm_count(dev);
     if (sms < 0) return sms;
+    const auto key = std::make_tuple(fn, dev, static_cast<int>(c.threads), smem);
     int fit = 0;
     {
         std::lock_guard<std::mutex> lk(g_occ_mu);
-        auto it = g_occ.find(std::make_tuple(fn, dev, static_cast<int>(c.threads), smem));
+        auto it = g_occ.find(key);
         if (it != g_occ.end()) fit = it->second;
     }
     if (fit == 0) {
+        const int st = ensure_smem_attr(fn, dev, smem);
+        if (st != AES_OK) return st;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, fn, c.threads, smem) != cudaSuccess) {
             (void)cudaGetLastError();
             return AES_E_CUDA;
         }
         std::lock_guard<std::mutex> lk(g_occ_mu);
-        g_occ[std::make_tuple(fn, dev, static_cast<int>(c.threads), smem)] = fit;
+        g_occ[key] = fit;
     }
     if (fit <= 0) return AES_E_CONFIG;
     const int per_sm = c.ctas_per_sm > 0 && c.ctas_per_sm < fit ? c.ctas_per_sm : fit;
@@ -157,11 +162,9 @@ int launch_ecb(int dir, const uint32_t *rk, int nr, const uint8_t *in, uint8_t *
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
     const uint32_t smem = ecb_smem_bytes(dir, c);
-    int st = ensure_smem_attr(fn, dev, smem);
-    if (st != AES_OK) return st;
     int grid = 0;
-    st = persistent_grid(fn, dev, c, smem,
-                         static_cast<unsigned long long>(c.threads) * c.blocks_per_thread, nblocks, &grid);
+    int st = persistent_grid(fn, dev, c, smem,
+                             static_cast<unsigned long long>(c.threads) * c.blocks_per_thread, nblocks, &grid);
     if (st != AES_OK) return st;
     EcbArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);

@@ -311,10 +311,8 @@ int launch_mode(const void *fn, int dir, const aes_launch_cfg &c, size_t nblocks
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
     const uint32_t smem = table_smem_bytes(dir, c.layout);
-    int st = ensure_smem_attr(fn, dev, smem);
-    if (st != AES_OK) return st;
     int grid = 0;
-    st = persistent_grid(fn, dev, c, smem, static_cast<unsigned long long>(c.threads), nblocks, &grid);
+    int st = persistent_grid(fn, dev, c, smem, static_cast<unsigned long long>(c.threads), nblocks, &grid);
     if (st != AES_OK) return st;
     set(grid);
     void *params[] = {&args};

@@ -237,14 +237,17 @@ aes_launch_cfg default_cfg(int dir, int /*nrounds*/, size_t nblocks) {
 }
 
 aes_launch_cfg tuned_or_default_cfg(int dir, int nrounds, size_t nblocks) {
-    const EcbKey key = ecb_key(dir, nrounds, nblocks);
+    bool any;
     {
         std::lock_guard<std::mutex> lk(g_mu);
         load_env_locked();
-        if (!g_ecb.empty()) {
-            auto it = g_ecb.find(key);
-            if (it != g_ecb.end()) return it->second;
-        }
+        any = !g_ecb.empty();
+    }
+    if (any) {  // the key takes the device's model: not looked up for nothing
+        const EcbKey key = ecb_key(dir, nrounds, nblocks);
+        std::lock_guard<std::mutex> lk(g_mu);
+        auto it = g_ecb.find(key);
+        if (it != g_ecb.end()) return it->second;
     }
     return default_cfg(dir, nrounds, nblocks);
 }
