@@ -43,6 +43,7 @@
 #include <cuda_runtime.h>
 
 #include "aes_tables.h"
+#include "bitslice.cuh"
 #include "bounds.cuh"
 
 namespace aesgb {
@@ -370,6 +371,61 @@ __device__ __forceinline__ void final_round(const TabT &tab, uint32_t (&s)[4], c
     for (int j = 0; j < 4; ++j) s[j] = t[j];
 }
 
+// The last round of encryption on two states without lookups: ShiftRows by byte
+// permutes (rows 1 and 3 by one column, then rows 2 and 3 by two), the 32 bytes
+// transposed into eight bit planes, the S-box circuit of the constant-time
+// kernel on whole planes, and back.  It takes 156 logic operations and 24
+// multiplications where the lookups take 32 wavefronts and 64 logic operations,
+// so it pays only as far as the logic pipe has room beside the lookups.
+__device__ __forceinline__ void transpose_bytes(uint32_t (&w)[8]) {
+    uint32_t m = 0x0F0F0F0Fu;
+#pragma unroll
+    for (int s = 4; s > 0; s >>= 1, m ^= (m << s))
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (!(k & s)) bs::exchange_bits(w[k], w[k + s], s, m);
+}
+
+template <class Key>
+__device__ __forceinline__ void final_round_logic(uint32_t (&a)[4], uint32_t (&b)[4], const Key &k, int kw) {
+    uint32_t p[8];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const uint32_t(&s)[4] = q ? b : a;
+        uint32_t t[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = __byte_perm(s[j], s[(j + 1) & 3], 0x7250u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[4 * q + j] = __byte_perm(t[j], t[(j + 2) & 3], 0x7610u);
+    }
+    transpose_bytes(p);
+    uint32_t in[16];  // planes; no key inputs
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        in[i] = p[i];
+        in[8 + i] = 0u;
+    }
+    bs::run<bsc::k_sbox_enc>(in, p);  // S(x) + 63
+    transpose_bytes(p);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t key = k(kw + j) ^ 0x63636363u;
+        a[j] = p[j] ^ key;
+        b[j] = p[4 + j] ^ key;
+    }
+}
+
+// Whether a kernel takes the last round of half its blocks without lookups.
+// With R4 tables and four blocks per thread the data pipe is 97 % busy and the
+// logic pipe 76 %; one pair of the four moves both to about 94 %.  AES-128
+// encryption, 512 threads: 256 MiB 287.9 -> 283.4 us, 1 GiB 1,144 -> 1,120 us.
+// Both pairs: 294 us at 256 MiB (the logic pipe binds); two blocks per thread,
+// one pair: 285.4; every second pass: 311 (divergent code paths share no
+// instruction cache).  Decryption (85 gates) 292.2 -> 287.8, no better than R2
+// with one block per thread (287.6), and R2's rotations leave no room.
+template <int DIR, int NB, int LAYOUT>
+constexpr bool kLogicHalf = DIR == kEncrypt && NB == 4 && LAYOUT == kLayoutR4;
+
 // Key accessor over the kernel-parameter round keys (constant bank).
 struct ParamKey {
     const uint32_t *w;
@@ -384,25 +440,27 @@ __device__ __forceinline__ uint32_t lookup_t(const TabT &tab, int t, uint32_t s,
     return pair_rotate<TabT>() && t >= 2 ? __byte_perm(v, 0u, 0x1032u) : v;
 }
 
-// Rounds R0..NR on NB states.
-template <int DIR, int NR, int NB, int R0, class TabT, class Key>
+// Rounds R0..NR on NB states; LOGIC: the last round of the first two states
+// without lookups.
+template <int DIR, int NR, int NB, int R0, bool LOGIC = false, class TabT, class Key>
 __device__ __forceinline__ void cipher_rounds(const TabT &tab, const Key &k, uint32_t (&s)[NB][4]) {
 #pragma unroll
     for (int r = R0; r < NR; ++r)
 #pragma unroll
         for (int i = 0; i < NB; ++i) full_round<DIR>(tab, s[i], k, 4 * r);
 #pragma unroll
-    for (int i = 0; i < NB; ++i) final_round<DIR>(tab, s[i], k, 4 * NR);
+    for (int i = LOGIC ? 2 : 0; i < NB; ++i) final_round<DIR>(tab, s[i], k, 4 * NR);
+    if constexpr (LOGIC) final_round_logic(s[0], s[1], k, 4 * NR);
 }
 
 // Full cipher (encrypt) or equivalent inverse cipher (decrypt) on NB states.
-template <int DIR, int NR, int NB, class TabT, class Key>
+template <int DIR, int NR, int NB, bool LOGIC = false, class TabT, class Key>
 __device__ __forceinline__ void cipher_states(const TabT &tab, const Key &k, uint32_t (&s)[NB][4]) {
 #pragma unroll
     for (int i = 0; i < NB; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) s[i][j] ^= k(j);
-    cipher_rounds<DIR, NR, NB, 1>(tab, k, s);
+    cipher_rounds<DIR, NR, NB, 1, LOGIC>(tab, k, s);
 }
 
 // Programmatic dependent launch.  The host launches the single-buffer kernels
@@ -467,7 +525,7 @@ __global__ void __launch_bounds__(max_threads_for(NB, LAYOUT), 1)
         for (int i = 0; i < NB; ++i) {
             s[i][0] = cur[i].x; s[i][1] = cur[i].y; s[i][2] = cur[i].z; s[i][3] = cur[i].w;
         }
-        cipher_states<DIR, NR, NB>(tab, key, s);
+        cipher_states<DIR, NR, NB, kLogicHalf<DIR, NB, LAYOUT>>(tab, key, s);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const unsigned long long b = base + lane + 32ull * i;

@@ -311,6 +311,14 @@ AESGB_HD uint32_t shl_mul(uint32_t x, int s) {
 #endif
 }
 
+// Swaps the bits of x under ~m, moved up by s, with those of y under m: after
+// it bit positions b (under m) and b + s of the pair hold x and y side by side.
+AESGB_HD void exchange_bits(uint32_t &x, uint32_t &y, int s, uint32_t m) {
+    const uint32_t u = x, v = y;
+    x = lop3<0xD8>(u, shl_mul(v, s), ~m);  // ~m ? (v << s) : u
+    y = lop3<0xD8>(v, u >> s, m);          //  m ? (u >> s) : v
+}
+
 AESGB_HD void transpose32(uint32_t *a) {
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
@@ -331,9 +339,7 @@ AESGB_HD void transpose32(uint32_t *a) {
 #pragma unroll
         for (int k = 0; k < 32; ++k) {
             if (k & s) continue;  // k runs over the words whose partner is k + s
-            const uint32_t x = a[k], y = a[k + s];
-            a[k] = lop3<0xD8>(x, shl_mul(y, s), ~m);     // ~m ? (y << s) : x
-            a[k + s] = lop3<0xD8>(y, x >> s, m);         //  m ? (x >> s) : y
+            exchange_bits(a[k], a[k + s], s, m);
         }
     }
 }

@@ -208,32 +208,35 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 // Untuned choice, by blocks per SM.  From 1,024 up one CTA of 1,024 threads per
 // SM, one block per thread: 32 warps keep the data pipe full and the unit of
 // 512 bytes divides evenly.  R4 tables encrypt; R2 decrypts, whose 128 KiB fill
-// faster than R4's 160, up to 16,384, from where the fill does not count.
+// faster than R4's 160 and which has fewer bank conflicts there.
 // From 128 up R2, 512 threads, as many CTAs as fit; below that 256 threads x 2
 // blocks: few, small CTAs, so that a stream of short launches finds room.
 // Replayed graph, against 256 threads x 2 blocks up to 16,384 blocks per SM:
 //   AES-128 encryption  2 MiB 5.4 -> 4.2 us, 4 MiB 7.1 -> 6.4, 16 MiB 21.0 ->
-//   19.65, 32 MiB 38.8 -> 37.5; 128 MiB (2 blocks per thread) 145.5 -> 144.9
+//   19.65, 32 MiB 38.8 -> 37.5
 //   AES-256 decryption  4 MiB 8.8 -> 8.6 us, 16 MiB 27.8 -> 26.9, 32 MiB 52.2 -> 51.6
+// Large buffers: from 49,152 blocks per SM (114 MiB) encryption takes four blocks
+// per thread, 512 threads, the form that keeps half of its last rounds off the
+// data pipe (kLogicHalf); its unit of 2 KiB costs more at the end of shorter
+// launches.  1,024 x 1 / 512 x 4, us:
+//   AES-128  64 MiB 74.3 / 74.5, 128 MiB 145.6 / 144.7, 1 GiB 1,145 / 1,124
+//   AES-192  64 MiB 88.4 / 87.6, 128 MiB 173.9 / 170.7, 1 GiB 1,371 / 1,333
+//   AES-256  64 MiB 101.7 / 102.1, 128 MiB 200.8 / 201.1, 1 GiB 1,585 / 1,576
+// Decryption keeps its former R4, 1,024 threads x 2 blocks between 16,384 and
+// 32,768 blocks per SM, where the R2 form gains 0.4-2 % (64 MiB: AES-128 75.8 /
+// 74.3, AES-256 102.3 / 101.9); above, R2: 1 GiB AES-128 1,161 -> 1,142, AES-256
+// 1,587 -> 1,581.
 aes_launch_cfg default_cfg(int dir, int /*nrounds*/, size_t nblocks) {
     const int found = current_sms();
-    const size_t sms = static_cast<size_t>(found > 0 ? found : 152);
-    aes_launch_cfg c;
-    c.blocks_per_thread = 1;
-    if (nblocks >= sms * 1024) {
-        c.layout = dir == 0 || nblocks >= sms * 16384 ? AES_LAYOUT_R4 : AES_LAYOUT_R2;
-        c.threads = 1024;
-        c.ctas_per_sm = 1;
-        return c;
+    const size_t per_sm = nblocks / static_cast<size_t>(found > 0 ? found : 152);
+    if (per_sm < 128) return aes_launch_cfg{256, 2, AES_LAYOUT_R2, 0};
+    if (per_sm < 1024) return aes_launch_cfg{512, 1, AES_LAYOUT_R2, 0};
+    if (dir == 0) {
+        if (per_sm >= 49152) return aes_launch_cfg{512, 4, AES_LAYOUT_R4, 1};
+        return aes_launch_cfg{1024, 1, AES_LAYOUT_R4, 1};
     }
-    c.layout = AES_LAYOUT_R2;
-    c.threads = 512;
-    c.ctas_per_sm = 0;
-    if (nblocks < sms * 128) {
-        c.threads = 256;
-        c.blocks_per_thread = 2;
-    }
-    return c;
+    if (per_sm >= 16384 && per_sm < 32768) return aes_launch_cfg{1024, 2, AES_LAYOUT_R4, 1};
+    return aes_launch_cfg{1024, 1, AES_LAYOUT_R2, 1};
 }
 
 aes_launch_cfg tuned_or_default_cfg(int dir, int nrounds, size_t nblocks) {

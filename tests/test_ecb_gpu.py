@@ -346,3 +346,40 @@ def test_default_cfg_small_size_switches(orc, blocks_per_sm):
             cfg = aesgb.aes_ecb_get_cfg(direction, 12, n)
             got, ok = gpu_ecb(direction, key, data, guard=64)
             assert ok and np.array_equal(got, orc.ecb(direction, key, data, nthreads=16)), (n, direction, cfg)
+
+
+@pytest.mark.parametrize("keybits", [128, 192, 256])
+def test_last_round_without_lookups(orc, keybits):
+    """R4 encryption with four blocks per thread takes the last round of a
+    thread's first two blocks in logic: every place of a block in the unit of
+    128, partial units, in place, all byte values in every position."""
+    torch = torch_cuda()
+    key = wl.random_key(keybits, 16).tobytes()
+    cfg = aesgb.make_cfg(512, 4, aesgb.LAYOUT_R4, 1)
+    for n in (1, 31, 32, 33, 63, 64, 65, 95, 97, 127, 128, 129, 4099):
+        data = wl.random_bytes(16 * n, 17 + n)
+        got, ok = gpu_ecb(0, key, data, cfg=cfg, inplace=n % 2 == 0, guard=64)
+        assert ok and np.array_equal(got, orc.ecb(0, key, data, nthreads=8)), n
+    every = np.repeat(np.arange(256, dtype=np.uint8), 16)   # 256 blocks of one byte value each
+    got, ok = gpu_ecb(0, key, every, cfg=cfg, guard=64)
+    assert ok and np.array_equal(got, orc.ecb(0, key, every)), "byte values"
+
+
+@pytest.mark.parametrize("blocks_per_sm, direction", [(32768, 1), (49152, 0)])
+def test_default_cfg_large_size_switches(orc, blocks_per_sm, direction):
+    """The lines of the untuned choice for large buffers: both sides give what
+    one fixed configuration gives on the whole buffer, and the oracle's bytes
+    on its first and last 64 KiB."""
+    torch = torch_cuda()
+    edge = aesgb.aes_device_sm_count(torch.cuda.current_device()) * blocks_per_sm
+    key = wl.random_key(256, 18).tobytes()
+    enc, dec, nr = aesgb.aes_expand_key(256, key)
+    rk = enc if direction == 0 else dec
+    for n in (edge - 1, edge + 33):
+        x = torch.empty(16 * n, dtype=torch.uint8, device="cuda").random_(0, 256)
+        y, z = torch.empty_like(x), torch.empty_like(x)
+        (aesgb.aes_ecb_encrypt if direction == 0 else aesgb.aes_ecb_decrypt)(rk, nr, x, y, n)
+        aesgb.aes_ecb_crypt_cfg(direction, rk, nr, x, z, n, aesgb.make_cfg(256, 1, aesgb.LAYOUT_R2, 0))
+        assert torch.equal(y, z), n
+        for part in (slice(0, 65536), slice(16 * n - 65536, 16 * n)):
+            assert np.array_equal(y[part].cpu().numpy(), orc.ecb(direction, key, x[part].cpu().numpy())), (n, part)
