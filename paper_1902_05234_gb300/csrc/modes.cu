@@ -187,8 +187,12 @@ __global__ void __launch_bounds__(max_threads_for_nb(NB), 1) chain_dec_kernel(co
     const uint32_t lane = threadIdx.x & 31u;
     const unsigned long long n = a.nblocks;
     const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * (blockDim.x >> 5) * 32ull * NB;
-    unsigned long long base =
-        (static_cast<unsigned long long>(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32ull * NB;
+    // Slices go round the CTAs first, as in ecb_kernel, while they make at most
+    // eight rounds of the grid; with more, CTA by CTA: the block before a slice is
+    // then in another warp's lines of the same SM (197 MiB, R4: CBC 236.9 -> 234.4
+    // us at AES-128, 319.1 -> 316.5 at AES-256).
+    const unsigned long long wpc = blockDim.x >> 5, warp = threadIdx.x >> 5;
+    unsigned long long base = (n <= 8 * step ? warp * gridDim.x + blockIdx.x : blockIdx.x * wpc + warp) * 32ull * NB;
     Tab<LAYOUT, DIR>::fill(smem, threadIdx.x, blockDim.x);
     __syncthreads();
     griddep_release();
@@ -261,6 +265,7 @@ const void *ctr_kernel_ptr(int nr, int layout) {
 
 const void *cbc_dec_kernel_ptr(int nr, int layout) {
     AESGB_C(kChainCbc, 10, kLayoutR2) AESGB_C(kChainCbc, 12, kLayoutR2) AESGB_C(kChainCbc, 14, kLayoutR2)
+    AESGB_C(kChainCbc, 10, kLayoutR4) AESGB_C(kChainCbc, 12, kLayoutR4) AESGB_C(kChainCbc, 14, kLayoutR4)
     return nullptr;
 }
 
@@ -272,20 +277,20 @@ const void *cfb_dec_kernel_ptr(int nr, int layout) {
 
 namespace {
 
-// Launch shape of a mode: one CTA of 1,024 threads per SM from 1,024 blocks per
-// SM up, with R4 tables where the forward cipher runs (CTR, CFB) and R2 for the
-// inverse one; below that R2, 512 threads, as many CTAs as fit.  Before, one CTA
-// of 256 threads with R4 tables ran up to 16,384 blocks per SM (40 MiB): 8 warps,
-// too few to keep the data pipe full.  Replayed graph, AES-128, 16 MiB: CBC 26.5
-// -> 21.4 us, CFB 25.4 -> 20.9; 4 MiB: CBC 8.2 -> 7.2, CFB 7.8 -> 6.9.  256 MiB:
-// CBC 305.0 (R4) -> 304.7 (R2); the line itself at 2 MiB: 512 against 1,024
-// threads CBC 4.61 / 4.71 us, at 4 MiB 7.30 / 7.16.
-aes_launch_cfg mode_cfg(int dir, size_t nblocks) {
+// Launch shape of a mode: one CTA of 1,024 threads per SM with R4 tables from
+// 1,024 blocks per SM up; below that R2, 512 threads, as many CTAs as fit.
+// Before, one CTA of 256 threads with R4 tables ran up to 16,384 blocks per SM
+// (40 MiB): 8 warps, too few to keep the data pipe full.  Replayed graph,
+// AES-128, 16 MiB: CBC 27.4 -> 21.9 us, CFB 26.2 -> 21.5; 4 MiB: CBC 8.9 -> 8.0,
+// CFB 8.6 -> 7.5.  R2 instead of R4: 197 MiB CBC 235.0 / 234.4 us, CFB 235.5 /
+// 232.7.  The line itself: 512 against 1,024 threads CBC 4.61 / 4.71 us at 2 MiB,
+// 7.30 / 7.16 at 4 MiB.
+aes_launch_cfg mode_cfg(size_t nblocks) {
     int dev = 0;
     const int sms = current_device(&dev) == AES_OK ? sm_count(dev) : 0;
     const bool large = nblocks >= static_cast<size_t>(sms > 0 ? sms : 152) * 1024;
     aes_launch_cfg c;
-    c.layout = large && dir == kEncrypt ? AES_LAYOUT_R4 : AES_LAYOUT_R2;
+    c.layout = large ? AES_LAYOUT_R4 : AES_LAYOUT_R2;
     c.threads = large ? 1024 : 512;
     c.blocks_per_thread = 1;
     c.ctas_per_sm = 0;
@@ -334,7 +339,7 @@ int aes_ctr_crypt(const uint32_t *rk, int nrounds, const uint8_t *ctr0, const ui
     if (nblocks == 0) return AES_OK;
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
-    const aes_launch_cfg c = mode_cfg(kEncrypt, nblocks);
+    const aes_launch_cfg c = mode_cfg(nblocks);
     CtrArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);
@@ -358,7 +363,7 @@ int aes_cbc_decrypt(const uint32_t *rk_dec, int nrounds, const uint8_t *iv, cons
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
     if (in == out) return AES_E_OVERLAP;  // a block's ciphertext is still needed after its plaintext is written
-    const aes_launch_cfg c = mode_cfg(kDecrypt, nblocks);
+    const aes_launch_cfg c = mode_cfg(nblocks);
     CbcArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);
@@ -377,7 +382,7 @@ int aes_cfb_decrypt(const uint32_t *rk_enc, int nrounds, const uint8_t *iv, cons
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
     if (in == out) return AES_E_OVERLAP;  // as CBC: C_i is read again after P_i would overwrite it
-    const aes_launch_cfg c = mode_cfg(kEncrypt, nblocks);
+    const aes_launch_cfg c = mode_cfg(nblocks);
     CbcArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);
