@@ -134,7 +134,8 @@ static_assert(kPlanMaxCtas <= kPlanThreads, "one tile per thread");
 static_assert(sizeof(PlanTile) <= 8 * kPlanThreads, "tiles fit");
 
 // Cost of the per-message work (finding it, its round keys) in the unit of one
-// round of one pass: about half a pass.
+// round of one pass: about half a pass.  20,000 messages of 16 B to 16 KiB with
+// 2 / 6 / 12 / 20 / 30: 96.4 / 96.5 / 100.0 / 102.9 / 108.5 us.
 constexpr unsigned int kMsgCost = 6;
 
 // The work of one message: nothing for an invalid or empty one.
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) batch_place_kernel(const __gr
         __syncthreads();
         unsigned int te = 0;
         unsigned long long tc[2] = {0, 0};  // totals of these 1,024
-        for (unsigned int w = 0; w < kPlanThreads / 32; ++w) {
+        for (unsigned int w = 0; w < blockDim.x >> 5; ++w) {
             if (w == warp) {
                 e += te;
                 c[0] += tc[0];
@@ -723,7 +724,8 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
         st = launch_pdl(reinterpret_cast<const void *>(&batch_place_kernel), ctas, kPlanThreads, 0, params, s);
         if (st != AES_OK) return st;
     } else {
-        batch_place_kernel<<<1, kPlanThreads, 0, s>>>(pa);
+        // one thread per descriptor: fewer warps to start and to scan over
+        batch_place_kernel<<<1, (n + 31) / 32 * 32, 0, s>>>(pa);
         if (cudaGetLastError() != cudaSuccess) return AES_E_CUDA;
     }
     return launch_batch_kernel(desc, n, ws, c, dev, s);
