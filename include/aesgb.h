@@ -247,7 +247,8 @@ typedef struct aes_batch_cfg {
     int32_t threads;           /* threads per CTA (multiple of 32, <= 512: keys sit in registers)    */
     int32_t blocks_per_thread; /* 1, 2 or 4                                                           */
     int32_t chunk_passes;      /* a chunk is 32 * blocks_per_thread * chunk_passes blocks of a message;
-                                  a warp's share of work at a time is at most two of them          */
+                                  a warp takes one equal share of up to 16 of them, or segments of
+                                  two in larger batches                                            */
     int32_t ctas_per_sm;       /* 0 or 1 (the tables take most of the shared memory)                */
     int32_t layout_enc;        /* table layout of the encryption phase and of the decryption      */
     int32_t layout_dec;        /* phase (aes_layout; section 4.2): the pairs R4/R2

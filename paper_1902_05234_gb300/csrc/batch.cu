@@ -12,11 +12,11 @@
 //                    cost is Nr for each pass of 32 * blocks_per_thread blocks
 //                    (what one warp ciphers at a time) plus kMsgCost for its key.
 //  batch  (persistent, one CTA per SM)  each direction's cost range is cut into
-//                    equal segments, one per warp when the batch is small, at
-//                    most chunk_passes passes each when it is large; a warp
-//                    starts with the segment of its own index and takes further
-//                    ones from an atomic counter.  A segment is walked message
-//                    by message: the first is found by a warp-wide 32-ary search
+//                    equal segments, one per warp up to 16 * chunk_passes passes
+//                    each, and into segments of 2 * chunk_passes (short ones at
+//                    the end) when the batch is larger; a warp starts with the
+//                    segment of its own index and takes further ones from an
+//                    atomic counter.  A segment is walked message by message: the first is found by a warp-wide 32-ary search
 //                    in start[], then each lane resolves one of the next 32
 //                    messages, and the warp ciphers them in turn with the next
 //                    message's round keys and first blocks already on their way.
@@ -138,23 +138,22 @@ static_assert(sizeof(PlanTile) <= 8 * kPlanThreads, "tiles fit");
 // 2 / 6 / 12 / 20 / 30: 96.4 / 96.5 / 100.0 / 102.9 / 108.5 us.
 constexpr unsigned int kMsgCost = 6;
 
-// The work of one message: nothing for an invalid or empty one.
-struct MsgWork {
-    unsigned long long cost, chunks;
-};
-__host__ __device__ inline MsgWork msg_work(unsigned long long nblocks, int nr, unsigned int pass_blocks,
-                                            unsigned int chunk_blocks) {
-    if (nblocks == 0) return {0ull, 0ull};
-    return {(nblocks + pass_blocks - 1) / pass_blocks * static_cast<unsigned int>(nr) + kMsgCost,
-            (nblocks + chunk_blocks - 1) / chunk_blocks};
+// Cost of one message, in passes of 2^pass_shift blocks; nothing for an empty one.
+__host__ __device__ inline unsigned long long msg_cost(unsigned long long nblocks, int nr, int pass_shift) {
+    if (nblocks == 0) return 0ull;
+    return (((nblocks - 1) >> pass_shift) + 1) * static_cast<unsigned int>(nr) + kMsgCost;
 }
+
+// log2 of the blocks of a pass, 32 * blocks_per_thread (1, 2 or 4).
+inline int pass_shift(const aes_batch_cfg &c) { return 5 + c.blocks_per_thread / 2; }
 
 struct PlanArgs {
     const aes_desc *desc;
     void *ws;
     int32_t *status;
     int n, per_cta;  // per_cta: descriptors of one CTA, a multiple of kPlanThreads
-    unsigned int pass_blocks, chunk_blocks;
+    int pass_shift;
+    unsigned int chunk_blocks;
 };
 
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
@@ -189,9 +188,8 @@ __device__ __forceinline__ PlanTile desc_tile(const aes_desc &d, int st, const P
     const bool ok = st == AES_OK;
     t.n_bad = !ok;
     t.n_enc = !ok || d.dir == 0;
-    const MsgWork w = ok ? msg_work(d.nblocks, d.nrounds, a.pass_blocks, a.chunk_blocks) : MsgWork{0ull, 0ull};
-    t.cost[t.n_enc ? 0 : 1] = w.cost;
-    t.chunks[t.n_enc ? 0 : 1] = w.chunks;
+    t.cost[t.n_enc ? 0 : 1] = ok ? msg_cost(d.nblocks, d.nrounds, a.pass_shift) : 0ull;
+    t.chunks[t.n_enc ? 0 : 1] = ok ? (d.nblocks + a.chunk_blocks - 1) / a.chunk_blocks : 0ull;
     return t;
 }
 
@@ -588,13 +586,17 @@ __device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, 
 }
 
 // Segments of a direction of total cost c on W warps: one equal share for each
-// warp while that is at most `most`; above, long ones and at the end (an eighth
-// of the whole, at most half a long one per warp) short ones, so that the
-// counter evens out the end.
+// warp while that is at most 8 * `most`; above, long ones of `most` and at the
+// end (an eighth of the whole, at most half a long one per warp) short ones, so
+// that the counter evens out the end.  A few long segments per warp are the
+// worst of both: a warp that takes one more than the others ends late.  Equal
+// shares up to 1, 4, 8, 16 * most: 4,096 messages of up to 1 MiB 587 / 530 / 531
+// / 531 us, 1,000 of up to 4 MiB 522 / 472 / 472 / 472, 2,000 of them through the
+// server 1,259 / 1,198 / 1,196 / 1,200.
 __device__ __forceinline__ Segments cut(unsigned long long c, unsigned int W, unsigned int most) {
     Segments s;
     const unsigned long long share = (c + W - 1) / W;
-    if (share <= most) {
+    if (share <= 8ull * most) {
         s.len = s.tail = share > 14 ? share : 14;  // at least a pass
         s.n = s.n_long = (c + s.len - 1) / s.len;
         return s;
@@ -614,12 +616,12 @@ constexpr int kBatchMaxThreads = 512;  // up to 128 registers: round keys live i
 // Bound: the L1TEX data pipe (the lookups) for large batches, 93-96 % busy; with
 // small messages the latencies in front of each one (its descriptor, keys and
 // first blocks), which is why the next message's are always under way, and why
-// a batch that gives a warp less than two chunks is cut into equal shares
-// instead of whole chunks.  Against one chunk of one message at a time, found by
+// a batch that gives a warp up to 16 chunks is cut into equal shares instead of
+// whole chunks.  Against one chunk of one message at a time, found by
 // a search each, behind a one-CTA plan: 20,000 messages of 16 B to 16 KiB 217 ->
-// 97 us (plan 87 -> about 9), 2,000 of them 64 -> 31, 20 of them 38 -> 12; 2,000
-// of up to 4 MiB 908 -> 893 us (kernel and plan), 4,096 of up to 16 MiB (5.2 GB)
-// 6,689 -> 6,640.  With 512 threads and the 44 to 60 key words in registers a
+// 97 us (plan 87 -> about 9), 2,000 of them 64 -> 31, 20 of them 38 -> 10.5;
+// 2,000 of up to 4 MiB 908 -> 884 us (kernel and plan), 4,096 of up to 16 MiB
+// (5.2 GB) 6,669 -> 6,650.  With 512 threads and the 44 to 60 key words in registers a
 // thread has one block in flight; two measured 20 % slower.
 template <int NB, int LE, int LD>
 __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_kernel(const __grid_constant__ BatchArgs a) {
@@ -712,7 +714,7 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
     pa.ws = ws;
     pa.status = status;
     pa.n = n;
-    pa.pass_blocks = static_cast<unsigned int>(32 * c.blocks_per_thread);
+    pa.pass_shift = pass_shift(c);
     pa.chunk_blocks = batch_chunk_blocks(c);
     const int tiles = (n + kPlanThreads - 1) / kPlanThreads, per = (tiles + kPlanMaxCtas - 1) / kPlanMaxCtas;
     pa.per_cta = per * kPlanThreads;
@@ -734,36 +736,34 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
 // ---------------------------------------------------------------------------
 // host-side planning (for callers that know their batch: the server)
 // ---------------------------------------------------------------------------
-// Writes into a HOST buffer of batch_plan_bytes(n) bytes exactly what the plan
-// kernels would write into that part of the workspace for these descriptors,
-// which must all be valid (check_desc): encryptions first in input order, then
-// decryptions; start[] the exclusive prefix of the costs; counters 0.
+// Writes into a HOST buffer of batch_plan_bytes(n) bytes what the plan kernels
+// would write into that part of the workspace for these descriptors, which must
+// all be valid (check_desc): encryptions first in input order, then decryptions;
+// start[] the exclusive prefix of the costs; counters 0.  The chunk totals, which
+// the batch kernel does not read, stay 0.
 void plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host) {
     const WsView v = ws_view(ws_host, n);
-    const unsigned int pass_blocks = static_cast<unsigned int>(32 * c.blocks_per_thread), chunk_blocks = batch_chunk_blocks(c);
+    const int shift = pass_shift(c);
     BatchHeader h{};
     unsigned long long run = 0;
     int pos = 0;
     for (int dir = 0; dir < 2; ++dir) {
         for (int i = 0; i < n; ++i)
             if (desc[i].dir == dir) {
-                const MsgWork w = msg_work(desc[i].nblocks, desc[i].nrounds, pass_blocks, chunk_blocks);
                 v.order[pos] = static_cast<uint32_t>(i);
                 v.start[pos] = run;
-                run += w.cost;
-                h.total_chunks += w.chunks;
+                run += msg_cost(desc[i].nblocks, desc[i].nrounds, shift);
                 ++pos;
             }
         if (dir == 0) {
             h.n_enc = static_cast<unsigned int>(pos);
             h.enc_cost = run;
-            h.enc_chunks = h.total_chunks;
         }
     }
     v.start[n] = run;
     h.total_cost = run;
     h.n = static_cast<unsigned int>(n);
-    h.chunk_blocks = chunk_blocks;
+    h.chunk_blocks = batch_chunk_blocks(c);
     *v.hdr = h;
 }
 
