@@ -206,8 +206,8 @@ def test_batch_graph_replay_and_library_workspace(orc):
 
 
 def test_batch_many_tiny_messages(orc):
-    """20,000 messages of 16..256 bytes: the plan kernel scans 20 tiles of
-    1,024 descriptors and the 32-ary search runs over 20,000 positions."""
+    """20,000 messages of 16..256 bytes: the plan takes 20 CTAs of 1,024
+    descriptors and the 32-ary search runs over 20,000 positions."""
     torch = torch_cuda()
     g = wl.rng(12)
     n = 20_000

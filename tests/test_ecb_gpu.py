@@ -46,11 +46,10 @@ def test_edge_sizes_default_cfg(orc, keybits, direction):
 
 
 def test_default_cfg_both_sides_of_the_size_switch(orc):
-    """The untuned configuration switches from the small-buffer choice (R2
-    tables, 256 threads x 2 blocks, three CTAs per SM) to the large-buffer one
-    (R4, 1,024 threads x 2 blocks, one CTA per SM) at 16,384 blocks per SM.
-    Buffers just below and above the switch, both directions, against the
-    oracle."""
+    """The untuned configuration for decryption switches from R2 tables with
+    one block per thread to R4 with two (1,024 threads, one CTA per SM) at
+    16,384 blocks per SM.  Buffers just below and above the switch, both
+    directions, against the oracle."""
     torch = torch_cuda()
     sms = aesgb.aes_device_sm_count(torch.cuda.current_device())
     key = wl.random_key(128, 12).tobytes()
