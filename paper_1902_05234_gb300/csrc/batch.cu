@@ -16,10 +16,11 @@
 //                    each, and into segments of 2 * chunk_passes (short ones at
 //                    the end) when the batch is larger; a warp starts with the
 //                    segment of its own index and takes further ones from an
-//                    atomic counter.  A segment is walked message by message: the first is found by a warp-wide 32-ary search
-//                    in start[], then each lane resolves one of the next 32
-//                    messages, and the warp ciphers them in turn with the next
-//                    message's round keys and first blocks already on their way.
+//                    atomic counter.  A segment is walked message by message:
+//                    the first is found by a warp-wide 32-ary search in start[],
+//                    then each lane resolves one of the next 32 messages, and
+//                    the warp ciphers them in turn with the next message's round
+//                    keys and first blocks already on their way.
 //                    The CTA's T tables are filled for encryption first and
 //                    refilled once for decryption, between two CTA barriers that
 //                    every warp reaches; each phase's table layout is part of the
@@ -542,7 +543,8 @@ __device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, 
                 const unsigned long long first = j0 * kPass;
                 const unsigned long long end = j1 * kPass < d.nblocks ? j1 * kPass : d.nblocks;
                 take = j0 < j1;
-                take = take && AESGB_CHECK(d.dir == DIR && end <= d.nblocks && first < end && end - first <= seg.len * kPass);
+                take = take && AESGB_CHECK(d.dir == DIR && end <= d.nblocks && first < end &&
+                                           end - first <= seg.len * kPass);
                 e.in = reinterpret_cast<const uint4 *>(d.in) + first;
                 e.out = reinterpret_cast<uint4 *>(d.out) + first;
                 e.rk = d.rk;
