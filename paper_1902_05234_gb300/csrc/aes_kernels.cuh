@@ -417,7 +417,7 @@ __device__ __forceinline__ void final_round_logic(uint32_t (&a)[4], uint32_t (&b
 
 // Whether a kernel takes the last round of half its blocks without lookups.
 // With R4 tables and four blocks per thread the data pipe is 97 % busy and the
-// logic pipe 76 %; one pair of the four moves both to about 94 %.  AES-128
+// logic pipe 76 %; one pair of the four moves them to 94 and 86 %.  AES-128
 // encryption, 512 threads: 256 MiB 287.9 -> 283.4 us, 1 GiB 1,144 -> 1,120 us.
 // Both pairs: 294 us at 256 MiB (the logic pipe binds); two blocks per thread,
 // one pair: 285.4; every second pass: 311 (divergent code paths share no
