@@ -29,7 +29,7 @@ struct CtrArgs {
     unsigned long long nblocks;
     RoundKeys rk;
     unsigned long long ctr_hi, ctr_lo;  // first counter block as a 128-bit integer
-    uint32_t passes;                    // passes of 32 * NB blocks per unit: 1, 2, 4 or 8, at most 256 blocks
+    uint32_t passes;                    // passes of 32 * NB blocks per unit: 2, 4 or 8, at most 256 blocks
 };
 
 struct CbcArgs {
@@ -163,6 +163,34 @@ __global__ void __launch_bounds__(max_threads_for_nb(NB), 1) ctr_kernel(const __
     }
 }
 
+// Up to a block per thread and 1,024 per SM: no shared rounds.  What 256 blocks
+// share would be computed for a unit of 32, ahead of the unit's own rounds, and
+// the time of such a call is one warp's chain of rounds.  A stream of launches
+// (replayed graph), this kernel against the shared form with 512 threads and R2
+// tables: 64 KiB AES-128 3.43 -> 1.78 us, AES-256 4.18 -> 2.07; 1 MiB 4.56 ->
+// 2.79 and 5.67 -> 3.28; 2 MiB 4.62 -> 3.98.  At 2.5 MiB the shared form takes
+// over (4.95 against 5.04 us).
+template <int NR, int LAYOUT>
+__global__ void __launch_bounds__(max_threads_for_nb(1), 1) ctr_small_kernel(const __grid_constant__ CtrArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t lane = threadIdx.x & 31u;
+    const unsigned long long step = static_cast<unsigned long long>(gridDim.x) * blockDim.x;
+    Tab<LAYOUT, kEncrypt>::fill(smem, threadIdx.x, blockDim.x);
+    __syncthreads();
+    griddep_release();
+    griddep_wait();  // global memory only after this (see aes_kernels.cuh)
+    const Tab<LAYOUT, kEncrypt> tab(smem, lane);
+    const ParamKey key{a.rk.w};
+    for (unsigned long long b = static_cast<unsigned long long>(blockIdx.x) * blockDim.x + threadIdx.x; b < a.nblocks;
+         b += step) {
+        const uint4 v = ld_block(a.in + b);
+        uint32_t s[1][4];
+        counter_state(a.ctr_hi, a.ctr_lo, b, s[0]);
+        cipher_states<kEncrypt, NR, 1>(tab, key, s);
+        st_block(a.out + b, make_uint4(v.x ^ s[0][0], v.y ^ s[0][1], v.z ^ s[0][2], v.w ^ s[0][3]));
+    }
+}
+
 __device__ __forceinline__ uint4 shfl_up1(uint4 v) {
     return make_uint4(__shfl_up_sync(0xffffffffu, v.x, 1), __shfl_up_sync(0xffffffffu, v.y, 1),
                       __shfl_up_sync(0xffffffffu, v.z, 1), __shfl_up_sync(0xffffffffu, v.w, 1));
@@ -252,15 +280,17 @@ AESGB_BOUNDS_READER(modes)
 
 // One block per thread: two at 1,024 threads measured 0.2 % (CFB) to 2 % (CBC)
 // slower at 256 MiB, AES-128, two at 512 threads 1-4 %.
-#define AESGB_M(KERNEL, NR, L) \
-    if (nr == NR && layout == L) return reinterpret_cast<const void *>(&KERNEL<NR, 1, L>);
+#define AESGB_M(KERNEL, ...) return reinterpret_cast<const void *>(&KERNEL<__VA_ARGS__>)
 #define AESGB_C(MODE, NR, L) \
     if (nr == NR && layout == L) return reinterpret_cast<const void *>(&chain_dec_kernel<MODE, NR, 1, L>);
 
-const void *ctr_kernel_ptr(int nr, int layout) {
-    AESGB_M(ctr_kernel, 10, kLayoutR4) AESGB_M(ctr_kernel, 12, kLayoutR4) AESGB_M(ctr_kernel, 14, kLayoutR4)
-    AESGB_M(ctr_kernel, 10, kLayoutR2) AESGB_M(ctr_kernel, 12, kLayoutR2) AESGB_M(ctr_kernel, 14, kLayoutR2)
-    return nullptr;
+const void *ctr_kernel_ptr(int nr, bool shared) {
+    switch (nr) {
+    case 10: if (shared) AESGB_M(ctr_kernel, 10, 1, kLayoutR4); else AESGB_M(ctr_small_kernel, 10, kLayoutR4);
+    case 12: if (shared) AESGB_M(ctr_kernel, 12, 1, kLayoutR4); else AESGB_M(ctr_small_kernel, 12, kLayoutR4);
+    case 14: if (shared) AESGB_M(ctr_kernel, 14, 1, kLayoutR4); else AESGB_M(ctr_small_kernel, 14, kLayoutR4);
+    default: return nullptr;
+    }
 }
 
 const void *cbc_dec_kernel_ptr(int nr, int layout) {
@@ -271,27 +301,38 @@ const void *cbc_dec_kernel_ptr(int nr, int layout) {
 
 const void *cfb_dec_kernel_ptr(int nr, int layout) {
     AESGB_C(kChainCfb, 10, kLayoutR4) AESGB_C(kChainCfb, 12, kLayoutR4) AESGB_C(kChainCfb, 14, kLayoutR4)
-    AESGB_C(kChainCfb, 10, kLayoutR2) AESGB_C(kChainCfb, 12, kLayoutR2) AESGB_C(kChainCfb, 14, kLayoutR2)
     return nullptr;
 }
 
 namespace {
 
-// Launch shape of a mode: one CTA of 1,024 threads per SM with R4 tables from
-// 1,024 blocks per SM up; below that R2, 512 threads, as many CTAs as fit.
-// Before, one CTA of 256 threads with R4 tables ran up to 16,384 blocks per SM
-// (40 MiB): 8 warps, too few to keep the data pipe full.  Replayed graph,
-// AES-128, 16 MiB: CBC 27.4 -> 21.9 us, CFB 26.2 -> 21.5; 4 MiB: CBC 8.9 -> 8.0,
-// CFB 8.6 -> 7.5.  R2 instead of R4: 197 MiB CBC 235.0 / 234.4 us, CFB 235.5 /
-// 232.7.  The line itself: 512 against 1,024 threads CBC 4.61 / 4.71 us at 2 MiB,
-// 7.30 / 7.16 at 4 MiB.
-aes_launch_cfg mode_cfg(size_t nblocks) {
+size_t blocks_per_sm(size_t nblocks) {  // rounded up
     int dev = 0;
-    const int sms = current_device(&dev) == AES_OK ? sm_count(dev) : 0;
-    const bool large = nblocks >= static_cast<size_t>(sms > 0 ? sms : 152) * 1024;
+    const int found = current_device(&dev) == AES_OK ? sm_count(dev) : 0;
+    const size_t sms = static_cast<size_t>(found > 0 ? found : 152);
+    return nblocks / sms + (nblocks % sms != 0);
+}
+
+// Launch shape of a mode, by blocks per SM.  One CTA per SM with R4
+// tables and one block per thread, of as many warps as an SM's share has: 256
+// threads up to 256 blocks per SM, 1,024 from 1,024 up.  R4 tables keep a second
+// CTA off the SM, so a small call spreads over as many SMs as it has CTAs; with
+// R2 tables and 512 threads it sat on half as many, up to three CTAs to an SM,
+// and a launch of the stream could meet the one before it there.  Replayed
+// graph, AES-128, 512 threads with R2 -> this: CFB 64 KiB 2.72 -> 1.78 us, 1 MiB
+// 3.2 to 4.5 -> 2.88, 2 MiB 6.0 -> 4.15; CBC 64 KiB 2.74 -> 2.02, 0.5 MiB 2.75
+// -> 2.45.  One CTA of 256 threads at all sizes: CFB 16 MiB 26.2 us against 21.5.
+//
+// CBC between 256 and 1,024 blocks per SM: its decryption tables take 160 KiB in
+// R4, whose fill shows there.  R2, and 512 threads from 384 blocks per SM:
+// 0.75 MiB (352 threads) 2.63 us with R2, 2.80 with R4, 2.78 with 512 threads
+// and R2; 1 MiB 3.05 / 3.24 / 2.91.
+aes_launch_cfg mode_cfg(bool cbc, size_t per_sm) {
+    const size_t share = per_sm < 256 ? 256 : per_sm > 1024 ? 1024 : (per_sm + 31) / 32 * 32;
+    const bool r2 = cbc && per_sm > 256 && per_sm <= 1024;
     aes_launch_cfg c;
-    c.layout = large ? AES_LAYOUT_R4 : AES_LAYOUT_R2;
-    c.threads = large ? 1024 : 512;
+    c.layout = r2 ? AES_LAYOUT_R2 : AES_LAYOUT_R4;
+    c.threads = static_cast<int32_t>(r2 && per_sm > 384 ? 512 : share);
     c.blocks_per_thread = 1;
     c.ctas_per_sm = 0;
     return c;
@@ -302,11 +343,11 @@ aes_launch_cfg mode_cfg(size_t nblocks) {
 // last round of units is short.  AES-128, 1,024 threads (1 / 2 / 4 / 8 passes):
 // 4 MiB 6.9 / 6.75 / 6.9 / - us, 8 MiB 11.1 / 10.96 / 10.54 / -, 16 MiB 18.9 /
 // 18.6 / 18.6 / 18.4, 32 MiB - / 34.1 / 34.0 / 34.3, 256 MiB - / 253.1 / 249.9 /
-// 248.6.
+// 248.6.  (More than 1,024 blocks per SM: two passes at least.)
 uint32_t ctr_passes(const aes_launch_cfg &c, int grid, size_t nblocks) {
     const unsigned long long per_pass = static_cast<unsigned long long>(grid) * static_cast<unsigned int>(c.threads);
     const unsigned long long r = (nblocks + per_pass - 1) / per_pass;  // passes if every warp takes the same
-    return r > 32 ? 8u : r > 8 ? 4u : r > 4 ? 8u : r > 2 ? 4u : r > 1 ? 2u : 1u;
+    return r > 32 ? 8u : r > 8 ? 4u : r > 4 ? 8u : r > 2 ? 4u : 2u;
 }
 
 // Grid and launch of a mode kernel; `set` is called with the grid first.
@@ -339,7 +380,8 @@ int aes_ctr_crypt(const uint32_t *rk, int nrounds, const uint8_t *ctr0, const ui
     if (nblocks == 0) return AES_OK;
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
-    const aes_launch_cfg c = mode_cfg(nblocks);
+    const size_t per_sm = blocks_per_sm(nblocks);
+    const aes_launch_cfg c = mode_cfg(false, per_sm);
     CtrArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);
@@ -350,7 +392,7 @@ int aes_ctr_crypt(const uint32_t *rk, int nrounds, const uint8_t *ctr0, const ui
     for (int b = 8; b < 16; ++b) lo = (lo << 8) | ctr0[b];
     args.ctr_hi = hi;
     args.ctr_lo = lo;
-    return launch_mode(ctr_kernel_ptr(nrounds, c.layout), kEncrypt, c, nblocks, args, stream,
+    return launch_mode(ctr_kernel_ptr(nrounds, per_sm > 1024), kEncrypt, c, nblocks, args, stream,
                        [&](int grid) { args.passes = ctr_passes(c, grid, nblocks); });
 }
 
@@ -363,7 +405,7 @@ int aes_cbc_decrypt(const uint32_t *rk_dec, int nrounds, const uint8_t *iv, cons
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
     if (in == out) return AES_E_OVERLAP;  // a block's ciphertext is still needed after its plaintext is written
-    const aes_launch_cfg c = mode_cfg(nblocks);
+    const aes_launch_cfg c = mode_cfg(true, blocks_per_sm(nblocks));
     CbcArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);
@@ -382,7 +424,7 @@ int aes_cfb_decrypt(const uint32_t *rk_enc, int nrounds, const uint8_t *iv, cons
     st = check_buffers(in, out, nblocks);
     if (st != AES_OK) return st;
     if (in == out) return AES_E_OVERLAP;  // as CBC: C_i is read again after P_i would overwrite it
-    const aes_launch_cfg c = mode_cfg(nblocks);
+    const aes_launch_cfg c = mode_cfg(false, blocks_per_sm(nblocks));
     CbcArgs args;
     args.in = reinterpret_cast<const uint4 *>(in);
     args.out = reinterpret_cast<uint4 *>(out);

@@ -47,3 +47,27 @@ def gpu_ecb(direction, key, data: np.ndarray, cfg=None, inplace=False, guard=0):
         fill = 0xA5 if inplace else 0x5A
         ok = bool(np.all(host[:guard] == fill) and np.all(host[guard + data.size:] == fill))
     return out, ok
+
+
+def stream_us(call, launches=100, replays=9):
+    """Time of one call in a stream of back-to-back calls, in microseconds: a
+    graph of `launches` calls replayed, the shortest of `replays`.  `call` takes
+    the stream."""
+    torch = torch_cuda()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        call(s)                                               # one-time set-up stays outside the capture
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            for _ in range(launches):
+                call(torch.cuda.current_stream())
+    best = float("inf")
+    for _ in range(replays):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        graph.replay()
+        end.record()
+        end.synchronize()
+        best = min(best, start.elapsed_time(end) * 1e3 / launches)
+    return best

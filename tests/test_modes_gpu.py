@@ -6,7 +6,7 @@ import pytest
 
 from paper_1902_05234_gb300 import aesgb
 from paper_1902_05234_gb300 import workloads as wl
-from gpu_util import torch_cuda
+from gpu_util import stream_us, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -146,7 +146,7 @@ def test_cfb_roundtrip_with_oracle_encryption(orc):
 @pytest.mark.parametrize("passes", [1, 2, 4, 8, 9, 33])
 def test_ctr_units_start_anywhere_in_a_group(orc, passes):
     """The CTR kernel shares the first two rounds inside groups of 256 counter
-    blocks and cuts them into units of 1, 2, 4 or 8 passes by the buffer's size:
+    blocks and cuts them into units of 2, 4 or 8 passes by the buffer's size:
     sizes at the edge of each choice, counters that start at the first, second,
     middle and last block of a group, and one whose carry leaves the lower 64 bits."""
     torch = torch_cuda()
@@ -186,7 +186,8 @@ def test_ctr_units_start_anywhere_in_a_group(orc, passes):
 
 @pytest.mark.parametrize("more", [-1, 0, 33])
 def test_chained_modes_at_the_size_switch(orc, more):
-    """CBC and CFB decryption change their launch shape at 1,024 blocks per SM."""
+    """CBC decryption changes its tables and threads at 1,024 blocks per SM, CFB
+    decryption fills its CTAs there."""
     torch = torch_cuda()
     n = aesgb.aes_device_sm_count(torch.cuda.current_device()) * 1024 + more
     key = wl.random_key(192, 97).tobytes()
@@ -200,3 +201,49 @@ def test_chained_modes_at_the_size_switch(orc, more):
         torch.cuda.synchronize()
         got = y.cpu().numpy()
         assert np.array_equal(got[:16 * n], ref(key, iv, data)) and np.all(got[16 * n:] == 0x5A), (call.__name__, n)
+
+
+@pytest.mark.parametrize("per_sm", [256, 384, 1024])
+def test_small_launch_shapes(orc, per_sm):
+    """Below 1,024 blocks per SM a CTA has as many warps as its SM's share, CTR
+    runs without shared rounds, and CBC takes R2 tables from 256 and 512 threads
+    from 384: both sides of each line, the counter carrying out of its lower 64
+    bits and out of all 128."""
+    torch = torch_cuda()
+    sms = aesgb.aes_device_sm_count(torch.cuda.current_device())
+    key = wl.random_key(192, 99).tobytes()
+    enc, dec, nr = aesgb.aes_expand_key(192, key)
+    iv = wl.random_bytes(16, 99)
+    wrap64 = np.frombuffer(bytes([0x11] * 8) + bytes([0xFF] * 6) + b"\x80\x05", np.uint8)
+    wrap128 = np.frombuffer(bytes([0xFF] * 14) + b"\x80\x05", np.uint8)
+    for n in (per_sm * sms - 1, per_sm * sms, per_sm * sms + 33):
+        data = wl.random_bytes(16 * n, 100)
+        x = torch.from_numpy(data).cuda()
+        y = torch.full((16 * n + 64,), 0x5A, dtype=torch.uint8, device="cuda")
+        for call, rk, block, ref in ((aesgb.aes_ctr_crypt, enc, wrap64, orc.ctr), (aesgb.aes_ctr_crypt, enc, wrap128, orc.ctr),
+                                     (aesgb.aes_cbc_decrypt, dec, iv, orc.cbc_decrypt),
+                                     (aesgb.aes_cfb_decrypt, enc, iv, orc.cfb_decrypt)):
+            call(rk, nr, block, x, y, n)
+            got = y.cpu().numpy()
+            assert np.array_equal(got[:16 * n], ref(key, block, data)) and np.all(got[16 * n:] == 0x5A), (call.__name__, n)
+
+
+@pytest.mark.parametrize("kib", [64, 512])
+def test_small_calls_in_a_stream_spread_over_the_sms(kib):
+    """A small call's time in a stream of calls is one warp's chain: with 256
+    threads per CTA and one CTA per SM the three modes measure 0.95 to 1.25 of an
+    ECB launch of that shape (R4 tables).  CTAs of 512 threads that share SMs, or
+    a chain longer by CTR's shared rounds, measured 1.5 to 2.1 at 64 KiB and 1.25
+    to 1.9 at 512."""
+    torch = torch_cuda()
+    key = wl.random_key(128, 101).tobytes()
+    enc, dec, nr = aesgb.aes_expand_key(128, key)
+    iv = bytes(16)
+    n = kib * 64
+    x = torch.zeros(16 * n, dtype=torch.uint8, device="cuda")
+    y = torch.empty_like(x)
+    cfg = aesgb.make_cfg(256, 1, aesgb.LAYOUT_R4, 1)
+    for call, rk, direction in ((aesgb.aes_ctr_crypt, enc, 0), (aesgb.aes_cfb_decrypt, enc, 0), (aesgb.aes_cbc_decrypt, dec, 1)):
+        ecb = stream_us(lambda s: aesgb.aes_ecb_crypt_cfg(direction, rk, nr, x, y, n, cfg, s))
+        mode = stream_us(lambda s: call(rk, nr, iv, x, y, n, s))
+        assert mode <= 1.1 * ecb, (call.__name__, kib, mode, ecb)
