@@ -209,12 +209,20 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 // SM, one block per thread: 32 warps keep the data pipe full and the unit of
 // 512 bytes divides evenly.  R4 tables encrypt; R2 decrypts, whose 128 KiB fill
 // faster than R4's 160 and which has fewer bank conflicts there.
-// From 128 up R2, 512 threads, as many CTAs as fit; below that 256 threads x 2
-// blocks: few, small CTAs, so that a stream of short launches finds room.
 // Replayed graph, against 256 threads x 2 blocks up to 16,384 blocks per SM:
-//   AES-128 encryption  2 MiB 5.4 -> 4.2 us, 4 MiB 7.1 -> 6.4, 16 MiB 21.0 ->
-//   19.65, 32 MiB 38.8 -> 37.5
-//   AES-256 decryption  4 MiB 8.8 -> 8.6 us, 16 MiB 27.8 -> 26.9, 32 MiB 52.2 -> 51.6
+//   AES-128 encryption  4 MiB 7.1 -> 6.2 us, 16 MiB 21.3 -> 19.6, 32 MiB 38.8 -> 37.5
+//   AES-256 decryption  4 MiB 8.6 -> 8.3 us, 16 MiB 27.5 -> 26.7, 32 MiB 51.9 -> 51.3
+// Smaller buffers, whose time is one warp's chain.  Decryption: 256 threads x 2
+// blocks up to 512 blocks per SM, then 512 x 1, R2, as many CTAs as fit; AES-128
+// 1 MiB 2.72 / 2.77 us, 1.5 MiB 3.75 / 3.49, AES-256 0.5 MiB 3.02 / 3.12.
+// Encryption with two CTAs to an SM falls, at some sizes, into a pattern where
+// the CTAs of one launch of a stream meet those of the one before (0.5 MiB, two
+// captures of the same calls: 2.8 and 4.5 us), so it takes R4 tables, which let
+// one CTA on an SM: 256 threads x 1 up to 256 blocks per SM, and above 512 as
+// many warps as the SM's share has; between, where that pattern is not seen, 256
+// x 2, R2.  AES-128, 512 threads x 1 with R2 / these: 0.25 MiB 2.90 / 1.78 us,
+// 0.5 MiB 2.81 / 2.18, 1 MiB 2.82 / 2.53 (448 x 1, R4: 2.78), 1.5 MiB 4.24 / 3.40,
+// 2 MiB 5.65 / 3.96 (1,024 x 1, R4: 4.07).
 // Large buffers: from 49,152 blocks per SM (114 MiB) encryption takes four blocks
 // per thread, 512 threads, the form that keeps half of its last rounds off the
 // data pipe (kLogicHalf); its unit of 2 KiB costs more at the end of shorter
@@ -228,9 +236,15 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 // 1,587 -> 1,581.
 aes_launch_cfg default_cfg(int dir, int /*nrounds*/, size_t nblocks) {
     const int found = current_sms();
-    const size_t per_sm = nblocks / static_cast<size_t>(found > 0 ? found : 152);
-    if (per_sm < 128) return aes_launch_cfg{256, 2, AES_LAYOUT_R2, 0};
-    if (per_sm < 1024) return aes_launch_cfg{512, 1, AES_LAYOUT_R2, 0};
+    const size_t sms = static_cast<size_t>(found > 0 ? found : 152);
+    const size_t per_sm = nblocks / sms;
+    if (per_sm < 1024) {
+        const size_t share = per_sm + (nblocks % sms != 0);
+        if (dir == 0 && share <= 256) return aes_launch_cfg{256, 1, AES_LAYOUT_R4, 1};
+        if (share <= 512) return aes_launch_cfg{256, 2, AES_LAYOUT_R2, 0};
+        if (dir == 0) return aes_launch_cfg{static_cast<int32_t>((share + 31) / 32 * 32), 1, AES_LAYOUT_R4, 1};
+        return aes_launch_cfg{512, 1, AES_LAYOUT_R2, 0};
+    }
     if (dir == 0) {
         if (per_sm >= 49152) return aes_launch_cfg{512, 4, AES_LAYOUT_R4, 1};
         return aes_launch_cfg{1024, 1, AES_LAYOUT_R4, 1};

@@ -171,6 +171,21 @@ def test_default_cfg_is_valid():
             assert c.threads % 32 == 0 and c.blocks_per_thread in (1, 2, 4, 8)
 
 
+def test_small_encryptions_take_one_cta_per_sm():
+    """Untuned encryption below 1,024 blocks per SM: one CTA per SM, with a block
+    for every thread, except between 256 and 512 (152 SMs without a device)."""
+    import torch
+    sms = aesgb.aes_device_sm_count(0) if torch.cuda.is_available() else 152
+    aesgb.aes_tune_clear()
+    for n in (1, 4096, 256 * sms, 512 * sms + 1, 700 * sms, 1024 * sms - 1):
+        c = aesgb.aes_ecb_get_cfg(0, 10, n)
+        assert (c.layout, c.blocks_per_thread, c.ctas_per_sm) == (aesgb.LAYOUT_R4, 1, 1), (n, c)
+        assert c.threads >= 256 and (c.threads == 256 or c.threads * sms - n < 32 * sms) and -(-n // c.threads) <= sms, (n, c)
+    for n in (256 * sms + 1, 512 * sms):
+        c = aesgb.aes_ecb_get_cfg(0, 10, n)
+        assert (c.threads, c.blocks_per_thread, c.layout) == (256, 2, aesgb.LAYOUT_R2), (n, c)
+
+
 def test_tune_cache_file_roundtrip(tmp_path):
     """Tuned entries set by hand survive save / clear / load (host logic)."""
     aesgb.aes_tune_clear()

@@ -331,11 +331,11 @@ def test_even_shares_at_one_cta_per_sm(orc, direction):
             assert ok and np.array_equal(got, exp), (nb, n, "in place")
 
 
-@pytest.mark.parametrize("blocks_per_sm", [128, 1024])
+@pytest.mark.parametrize("blocks_per_sm", [128, 256, 512, 1024])
 def test_default_cfg_small_size_switches(orc, blocks_per_sm):
-    """The other two lines of the untuned choice (256 threads x 2 blocks, 512
-    threads, 1,024 threads): buffers just below, at and above each, both
-    directions, in units that go round the CTAs with a ragged last one."""
+    """The lines of the untuned choice below 1,024 blocks per SM, and a size inside
+    one of its ranges: buffers just below, at and above each, both directions, in
+    units that go round the CTAs with a ragged last one."""
     torch = torch_cuda()
     edge = aesgb.aes_device_sm_count(torch.cuda.current_device()) * blocks_per_sm
     key = wl.random_key(192, 14).tobytes()
