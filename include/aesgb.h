@@ -251,9 +251,9 @@ typedef struct aes_batch_cfg {
                                   two in larger batches                                            */
     int32_t ctas_per_sm;       /* 0 or 1 (the tables take most of the shared memory)                */
     int32_t layout_enc;        /* table layout of the encryption phase and of the decryption      */
-    int32_t layout_dec;        /* phase (aes_layout; section 4.2): the pairs R4/R2
-                                  (blocks_per_thread 1, 2 or 4), R4/R4 (the default), R2/R2 and
-                                  R1/R1 (1 or 2); another pair is AES_E_CONFIG                       */
+    int32_t layout_dec;        /* phase (aes_layout; section 4.2): the pairs R4/R4 (the default) and
+                                  R4/R2 (blocks_per_thread 1, 2 or 4), R2/R2 and R1/R1 (1 or 2);
+                                  another pair is AES_E_CONFIG                                       */
 } aes_batch_cfg;
 
 /* Bytes of DEVICE workspace a batch of n descriptors needs (plan header, the

@@ -660,13 +660,13 @@ uint32_t batch_smem_bytes(const aes_batch_cfg &c) {
 }
 
 // The compiled (blocks per thread, encryption layout, decryption layout)
-// combinations: the pair R4 / R2 at 1, 2 and 4 blocks per thread, and the pairs
-// R4 / R4 (the default), R2 / R2 and R1 / R1 at 1 and 2 (the tuner's range).
+// combinations: the pairs R4 / R4 (the default) and R4 / R2 at 1, 2 and 4 blocks
+// per thread, and the pairs R2 / R2 and R1 / R1 at 1 and 2 (the tuner's range).
 const void *batch_kernel_ptr(int nb, int le, int ld) {
 #define AESGB_BK(NB, LE, LD) \
     if (nb == NB && le == LE && ld == LD) return reinterpret_cast<const void *>(&batch_kernel<NB, LE, LD>);
     AESGB_BK(1, kLayoutR4, kLayoutR2) AESGB_BK(2, kLayoutR4, kLayoutR2) AESGB_BK(4, kLayoutR4, kLayoutR2)
-    AESGB_BK(1, kLayoutR4, kLayoutR4) AESGB_BK(2, kLayoutR4, kLayoutR4)
+    AESGB_BK(1, kLayoutR4, kLayoutR4) AESGB_BK(2, kLayoutR4, kLayoutR4) AESGB_BK(4, kLayoutR4, kLayoutR4)
     AESGB_BK(1, kLayoutR2, kLayoutR2) AESGB_BK(2, kLayoutR2, kLayoutR2)
     AESGB_BK(1, kLayoutR1, kLayoutR1) AESGB_BK(2, kLayoutR1, kLayoutR1)
 #undef AESGB_BK

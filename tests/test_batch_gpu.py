@@ -161,6 +161,20 @@ def test_batch_cfg_layout_pairs_refused_outside_the_compiled_set():
         assert e.value.status == -12, repr(cfg)
 
 
+@pytest.mark.parametrize("nb", [1, 2, 4])
+def test_default_batch_cfg_at_other_granularities(orc, nb):
+    """The default configuration with only its blocks per thread changed is taken
+    at 1, 2 and 4."""
+    torch = torch_cuda()
+    lengths, keybits, dirs = small_mix(90, hi=64 * 1024, seed=11)
+    b = DeviceBatch(torch, lengths, keybits, dirs, seed=9)
+    ws, nbytes = b.workspace()
+    cfg = aesgb.aes_batch_get_cfg(b.n)
+    cfg.blocks_per_thread = nb
+    aesgb.aes_ecb_batch_ws(b.desc_dev, b.n, ws, nbytes, cfg=cfg)
+    check_against_oracle(orc, b, b.output())
+
+
 def test_batch_every_cfg(orc):
     torch = torch_cuda()
     lengths, keybits, dirs = small_mix(150, hi=128 * 1024, seed=9)
