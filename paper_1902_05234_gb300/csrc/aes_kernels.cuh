@@ -415,16 +415,20 @@ __device__ __forceinline__ void final_round_logic(uint32_t (&a)[4], uint32_t (&b
     }
 }
 
-// Whether a kernel takes the last round of half its blocks without lookups.
-// With R4 tables and four blocks per thread the data pipe is 97 % busy and the
-// logic pipe 76 %; one pair of the four moves them to 94 and 86 %.  AES-128
-// encryption, 512 threads: 256 MiB 287.9 -> 283.4 us, 1 GiB 1,144 -> 1,120 us.
-// Both pairs: 294 us at 256 MiB (the logic pipe binds); two blocks per thread,
-// one pair: 285.4; every second pass: 311 (divergent code paths share no
-// instruction cache).  Decryption (85 gates) 292.2 -> 287.8, no better than R2
-// with one block per thread (287.6), and R2's rotations leave no room.
-template <int DIR, int NB, int LAYOUT>
-constexpr bool kLogicHalf = DIR == kEncrypt && NB == 4 && LAYOUT == kLayoutR4;
+// Whether a launch takes the last round of half its blocks without lookups.
+// With R4 tables, four blocks per thread and 512 threads the data pipe is 97 %
+// busy and the logic pipe 76 %; one pair of the four moves them to 94 and 86 %.
+// AES-128 encryption: 256 MiB 288.8 -> 284.7 us, 1 GiB 1,147 -> 1,127 us (below
+// 64 MiB up to 3 % slower; the default takes this shape from 114 MiB).  Both
+// pairs: 294 us at 256 MiB (the logic pipe binds); two blocks per thread, one
+// pair: 285.4; every second pass: 311 (divergent code paths share no instruction
+// cache).  With fewer warps the longer code costs more than the lookups it saves:
+// 256 threads, 256 MiB, AES-128 290.8 us without and 297.5 with, AES-256 401 and
+// 466.  Decryption (85 gates) 292.2 -> 287.8, no better than R2 with one block
+// per thread (287.6), and R2's rotations leave no room.
+constexpr bool logic_half(int nb, int layout, int threads) {
+    return nb == 4 && layout == kLayoutR4 && threads == 512;
+}
 
 // Key accessor over the kernel-parameter round keys (constant bank).
 struct ParamKey {
@@ -489,7 +493,7 @@ __device__ __forceinline__ void st_block(uint4 *p, uint4 v) { __stcs(p, v); }
 // that at one CTA per SM, measured 0-3 % slower than this (AES-128 encryption,
 // 1,024 threads: 4 MiB 6.84 -> 6.38 us, 8 MiB 11.3 -> 10.8, 16 MiB 20.0 -> 19.65).
 // ---------------------------------------------------------------------------
-template <int DIR, int NR, int NB, int LAYOUT>
+template <int DIR, int NR, int NB, int LAYOUT, bool LOGIC = false>
 __global__ void __launch_bounds__(max_threads_for(NB, LAYOUT), 1)
     ecb_kernel(const __grid_constant__ EcbArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -530,7 +534,7 @@ __global__ void __launch_bounds__(max_threads_for(NB, LAYOUT), 1)
         for (int i = 0; i < NB; ++i) {
             s[i][0] = cur[i].x; s[i][1] = cur[i].y; s[i][2] = cur[i].z; s[i][3] = cur[i].w;
         }
-        cipher_states<DIR, NR, NB, kLogicHalf<DIR, NB, LAYOUT>>(tab, key, s);
+        cipher_states<DIR, NR, NB, LOGIC>(tab, key, s);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const unsigned long long b = base + lane + 32ull * i;

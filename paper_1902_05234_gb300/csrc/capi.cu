@@ -81,9 +81,10 @@ void order_round_keys(int dir, const uint32_t *rk, int nr, RoundKeys *out) {
     }
 }
 
-const void *ecb_kernel_ptr(int dir, int nr, int nb, int layout) {
-    if (layout == AES_LAYOUT_R4_TMA) return ecb_kernel_tma(dir, nr, nb);
-    return dir == kEncrypt ? ecb_kernel_enc(nr, nb, layout) : ecb_kernel_dec(nr, nb, layout);
+const void *ecb_kernel_ptr(int dir, int nr, const aes_launch_cfg &c) {
+    if (c.layout == AES_LAYOUT_R4_TMA) return ecb_kernel_tma(dir, nr, c.blocks_per_thread);
+    return dir == kEncrypt ? ecb_kernel_enc(nr, c.blocks_per_thread, c.layout, c.threads)
+                           : ecb_kernel_dec(nr, c.blocks_per_thread, c.layout);
 }
 
 uint32_t ecb_smem_bytes(int dir, const aes_launch_cfg &c) {
@@ -157,7 +158,7 @@ int launch_pdl(const void *fn, int grid, int threads, uint32_t smem, void **para
 
 int launch_ecb(int dir, const uint32_t *rk, int nr, const uint8_t *in, uint8_t *out, size_t nblocks,
                const aes_launch_cfg &c, void *stream) {
-    const void *fn = ecb_kernel_ptr(dir, nr, c.blocks_per_thread, c.layout);
+    const void *fn = ecb_kernel_ptr(dir, nr, c);
     if (!fn) return AES_E_CONFIG;
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;

@@ -18,7 +18,12 @@ namespace aesgb {
 
 AESGB_BOUNDS_READER(ecb_enc)
 
-const void *ecb_kernel_enc(int nr, int nb, int layout) {
+const void *ecb_kernel_enc(int nr, int nb, int layout, int threads) {
+    if (logic_half(nb, layout, threads)) {
+        if (nr == 10) return reinterpret_cast<const void *>(&ecb_kernel<kEncrypt, 10, 4, kLayoutR4, true>);
+        if (nr == 12) return reinterpret_cast<const void *>(&ecb_kernel<kEncrypt, 12, 4, kLayoutR4, true>);
+        if (nr == 14) return reinterpret_cast<const void *>(&ecb_kernel<kEncrypt, 14, 4, kLayoutR4, true>);
+    }
     AESGB_NR(10)
     AESGB_NR(12)
     AESGB_NR(14)

@@ -7,8 +7,8 @@
 namespace aesgb {
 
 // Host stub of ecb_kernel<dir, nr, nb, layout>, or nullptr if that
-// combination is not compiled.
-const void *ecb_kernel_enc(int nr, int nb, int layout);
+// combination is not compiled (encryption: of the form for that many threads).
+const void *ecb_kernel_enc(int nr, int nb, int layout, int threads);
 const void *ecb_kernel_dec(int nr, int nb, int layout);
 
 // ecb_tma.cu: the TMA-staged variant (layout AES_LAYOUT_R4_TMA), its dynamic

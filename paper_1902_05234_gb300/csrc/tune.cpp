@@ -225,7 +225,7 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 // 2 MiB 5.65 / 3.96 (1,024 x 1, R4: 4.07).
 // Large buffers: from 49,152 blocks per SM (114 MiB) encryption takes four blocks
 // per thread, 512 threads, the form that keeps half of its last rounds off the
-// data pipe (kLogicHalf); its unit of 2 KiB costs more at the end of shorter
+// data pipe (logic_half); its unit of 2 KiB costs more at the end of shorter
 // launches.  1,024 x 1 / 512 x 4, us:
 //   AES-128  64 MiB 74.3 / 74.5, 128 MiB 145.6 / 144.7, 1 GiB 1,145 / 1,124
 //   AES-192  64 MiB 88.4 / 87.6, 128 MiB 173.9 / 170.7, 1 GiB 1,371 / 1,333

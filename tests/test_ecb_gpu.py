@@ -6,7 +6,7 @@ import pytest
 
 from paper_1902_05234_gb300 import aesgb
 from paper_1902_05234_gb300 import workloads as wl
-from gpu_util import gpu_ecb, torch_cuda
+from gpu_util import gpu_ecb, stream_us, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -362,6 +362,19 @@ def test_last_round_without_lookups(orc, keybits):
     every = np.repeat(np.arange(256, dtype=np.uint8), 16)   # 256 blocks of one byte value each
     got, ok = gpu_ecb(0, key, every, cfg=cfg, guard=64)
     assert ok and np.array_equal(got, orc.ecb(0, key, every)), "byte values"
+
+
+def test_four_blocks_per_thread_with_few_warps():
+    """256 threads x 4 blocks (R4, AES-256) have no issue slots to spare for a last
+    round in logic: within 5 % of 512 threads x 4 at 64 MiB (10 % over with it)."""
+    torch = torch_cuda()
+    enc, _, nr = aesgb.aes_expand_key(256, wl.random_key(256, 19).tobytes())
+    n = 1 << 22
+    x = torch.empty(16 * n, dtype=torch.uint8, device="cuda").random_(0, 256)
+    y = torch.empty_like(x)
+    few, full = (stream_us(lambda s: aesgb.aes_ecb_crypt_cfg(
+        0, enc, nr, x, y, n, aesgb.make_cfg(threads, 4, aesgb.LAYOUT_R4, 1), s), launches=20) for threads in (256, 512))
+    assert few <= 1.05 * full, (few, full)
 
 
 @pytest.mark.parametrize("blocks_per_sm, direction", [(32768, 1), (49152, 0)])
