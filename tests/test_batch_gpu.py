@@ -8,7 +8,7 @@ import pytest
 from paper_1902_05234_gb300 import aesgb
 from paper_1902_05234_gb300 import workloads as wl
 from batch_util import DeviceBatch
-from gpu_util import torch_cuda
+from gpu_util import stream_us, torch_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -312,3 +312,30 @@ def test_batch_plan_and_segment_edges(orc, n, invalid):
             if i not in exp:
                 exp[i] = orc.ecb(int(b.dirs[i]), b.keys[i], b.message(b.data, i))
             assert np.array_equal(got, exp[i]), (i, repr(cfg))
+
+
+@pytest.mark.parametrize("unused", ["empty", "invalid"])
+def test_batch_run_of_unused_descriptors_in_the_middle(orc, unused):
+    """20,000 descriptors of which the first 24 and the last 17 are messages: as
+    fast as with all messages in front (one warp that walks the run 32 descriptors
+    at a time takes 8 to 14 times as long), and the messages exact."""
+    torch = torch_cuda()
+    n, front, back = 20_000, 24, 17
+    g = wl.rng(14)
+    keybits, dirs = g.choice(np.array([128, 192, 256]), size=n), g.integers(0, 2, size=n)
+    times = []
+    for used in (np.r_[0:front, n - back:n], np.r_[0:front + back]):
+        lengths = np.zeros(n, np.int64)
+        lengths[used] = 16 * g.integers(1, 200, size=used.size)
+        if unused == "invalid":
+            lengths[lengths == 0] = 16
+        b = DeviceBatch(torch, lengths, keybits, dirs, seed=14)
+        bad = set(range(n)) - set(used.tolist()) if unused == "invalid" else set()
+        if bad:
+            b.table["nrounds"][sorted(bad)] = 11
+            b.upload()
+        ws, nbytes = b.workspace()
+        aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes)
+        check_against_oracle(orc, b, b.output(), skip=bad)
+        times.append(stream_us(lambda s: aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes, stream=s), launches=20))
+    assert times[0] <= 1.5 * times[1], times
