@@ -117,6 +117,12 @@ int aes_test_fail_allocs(int skip, int count);
  * AES_E_CONFIG with all three 0 in the release build.  DEVICE-synchronous. */
 int aes_debug_batch_coverage(unsigned long long *once, unsigned long long *repeated, unsigned long long *beyond);
 
+/* Debug build only: what the batch launches since the last call did.  *fills:
+ * times a CTA filled its tables; *counter: segments that a warp took from the
+ * work counter, beyond the one of its own index.  Clears both.  AES_E_CONFIG
+ * with both 0 in the release build.  DEVICE-synchronous. */
+int aes_debug_batch_counts(unsigned long long *fills, unsigned long long *counter);
+
 /* Failure-detection test hook: one warp of the TMA-staged encryption kernel
  * on nblocks (1..64) DEVICE blocks, with every mbarrier expecting 16 bytes
  * more than its bulk copy delivers.  The copies land, but no wait can finish:

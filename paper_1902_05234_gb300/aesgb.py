@@ -127,6 +127,7 @@ _SIGNATURES = {
     "aes_tma_selftest_timeout": (_i, [_vp, _vp, _sz, _vp]),
     "aes_debug_bounds_violations": (_i, [ctypes.POINTER(ctypes.c_ulonglong)]),
     "aes_debug_batch_coverage": (_i, [ctypes.POINTER(ctypes.c_ulonglong)] * 3),
+    "aes_debug_batch_counts": (_i, [ctypes.POINTER(ctypes.c_ulonglong)] * 2),
     "aes_ctr_crypt": (_i, [_vp, _i, _vp, _vp, _vp, _sz, _vp]),
     "aes_cbc_decrypt": (_i, [_vp, _i, _vp, _vp, _vp, _sz, _vp]),
     "aes_cfb_decrypt": (_i, [_vp, _i, _vp, _vp, _vp, _sz, _vp]),
@@ -498,6 +499,15 @@ def aes_debug_batch_coverage() -> tuple[int, int, int]:
     v = [ctypes.c_ulonglong() for _ in range(3)]
     _check(lib().aes_debug_batch_coverage(*[ctypes.byref(x) for x in v]), "aes_debug_batch_coverage")
     return v[0].value, v[1].value, v[2].value
+
+
+def aes_debug_batch_counts() -> tuple[int, int]:
+    """(fills, counter) of the debug build's batch launches since the last call
+    (AES_E_CONFIG in the release build): table fills of a CTA, and segments taken
+    from the work counter."""
+    v = [ctypes.c_ulonglong() for _ in range(2)]
+    _check(lib().aes_debug_batch_counts(*[ctypes.byref(x) for x in v]), "aes_debug_batch_counts")
+    return tuple(int(x.value) for x in v)
 
 
 def aes_tma_selftest_timeout(in_, out, nblocks: int, stream=None) -> None:

@@ -325,6 +325,7 @@ struct BatchArgs {
     const aes_desc *desc;
     void *ws;
     int n;
+    int first;  // the direction whose tables are filled ahead of the plan: kDecrypt only if no message encrypts
 };
 
 constexpr uint32_t kKeySlotBytes = 256;  // 60 words rounded up
@@ -363,6 +364,15 @@ __host__ __device__ constexpr uint32_t batch_table_bytes(int le, int ld) {
 constexpr unsigned int kTagChunks = 1u << 16;
 static __device__ unsigned int g_chunk_tag[kTagChunks];
 static __device__ unsigned long long g_chunk_tag_beyond;
+#endif
+
+#if defined(AESGB_BOUNDS_CHECK)
+// Debug build: what the batch launches did, for aes_debug_batch_counts.
+enum { kCountFills, kCountCounter, kCounts };
+static __device__ unsigned long long g_batch_counts[kCounts];
+#define AESGB_COUNT(WHICH) atomicAdd(&g_batch_counts[WHICH], 1ull)
+#else
+#define AESGB_COUNT(WHICH) ((void)0)
 #endif
 
 // Round keys of the current message held in registers for all its passes
@@ -520,6 +530,7 @@ __device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, 
     while (rel < seg.n) {
         unsigned long long ticket = 0;
         if (seg.n > W && lane == 0) ticket = atomicAdd(&v.hdr->next[DIR], 1ull);
+        if (rel >= W && lane == 0) AESGB_COUNT(kCountCounter);
         const unsigned long long lo = c_begin + seg.begin(rel), stop = c_begin + seg.begin(rel + 1);
         const unsigned long long hi = stop < c_end ? stop : c_end;
         p = find_message(v.start, p, p_end, lo, lane);
@@ -620,6 +631,11 @@ __device__ __forceinline__ Segments cut(unsigned long long c, unsigned int W, un
     return s;
 }
 
+template <int LAYOUT, int DIR> __device__ __forceinline__ void fill_tables(uint8_t *smem) {
+    Tab<LAYOUT, DIR>::fill(smem, threadIdx.x, blockDim.x);
+    if (threadIdx.x == 0) AESGB_COUNT(kCountFills);
+}
+
 constexpr int kBatchMaxThreads = 512;  // up to 128 registers: round keys live in registers
 
 // LE, LD: table layouts of the encryption and decryption phases.
@@ -641,7 +657,8 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_kernel(const __grid
     uint8_t *wslot = smem + batch_table_bytes(LE, LD) + (threadIdx.x >> 5) * kWarpSlotBytes;
     // launched behind the plan (programmatic dependent launch): the first fill
     // reads only constant tables and runs while the plan does
-    Tab<LE, kEncrypt>::fill(smem, threadIdx.x, blockDim.x);
+    if (a.first == kEncrypt) fill_tables<LE, kEncrypt>(smem);
+    else fill_tables<LD, kDecrypt>(smem);
     griddep_wait();
     __syncthreads();
     const unsigned long long E = v.hdr->enc_cost, T = v.hdr->total_cost;
@@ -655,9 +672,11 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_kernel(const __grid
     const Segments se = cut(E, W, most), sd = cut(T - E, W, most);
     if (blockIdx.x < se.n) batch_phase<kEncrypt, NB, LE>(a, v, smem, wslot, row + blockIdx.x, W, 0, E, 0, n_enc, se);
     if (back < sd.n) {
-        __syncthreads();  // every warp is done with the encryption tables
-        Tab<LD, kDecrypt>::fill(smem, threadIdx.x, blockDim.x);
-        __syncthreads();
+        if (a.first == kEncrypt) {
+            __syncthreads();  // every warp is done with the encryption tables
+            fill_tables<LD, kDecrypt>(smem);
+            __syncthreads();
+        }
         batch_phase<kDecrypt, NB, LD>(a, v, smem, wslot, row + back, W, E, T, n_enc, a.n, sd);
     }
 }
@@ -697,14 +716,15 @@ unsigned int batch_chunk_blocks(const aes_batch_cfg &c) {
 
 // The persistent kernel on a planned workspace; the plan is the kernel (or the
 // copy) before it in the stream.
-int launch_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_cfg &c, int dev, cudaStream_t s) {
+int launch_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_cfg &c, int first, int dev,
+                        cudaStream_t s) {
     const void *fn = batch_kernel_ptr(c.blocks_per_thread, c.layout_enc, c.layout_dec);
     const uint32_t smem = batch_smem_bytes(c);
     const int st = ensure_smem_attr(fn, dev, smem);
     if (st != AES_OK) return st;
     const int sms = sm_count(dev);
     if (sms < 0) return sms;
-    BatchArgs args{desc, ws, n};
+    BatchArgs args{desc, ws, n, first};
     void *params[] = {&args};
     return launch_pdl(fn, sms, c.threads, smem, params, s);
 }
@@ -741,7 +761,7 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
         batch_place_kernel<<<1, (n + 31) / 32 * 32, 0, s>>>(pa);
         if (cudaGetLastError() != cudaSuccess) return AES_E_CUDA;
     }
-    return launch_batch_kernel(desc, n, ws, c, dev, s);
+    return launch_batch_kernel(desc, n, ws, c, kEncrypt, dev, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -751,8 +771,8 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
 // would write into that part of the workspace for these descriptors, which must
 // all be valid (check_desc): encryptions first in input order, then decryptions;
 // start[] the exclusive prefix of the costs; counters 0.  The chunk totals, which
-// the batch kernel does not read, stay 0.
-void plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host) {
+// the batch kernel does not read, stay 0.  Returns how many messages encrypt.
+int plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host) {
     const WsView v = ws_view(ws_host, n);
     const int shift = pass_shift(c);
     BatchHeader h{};
@@ -776,17 +796,20 @@ void plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_
     h.n = static_cast<unsigned int>(n);
     h.chunk_blocks = batch_chunk_blocks(c);
     *v.hdr = h;
+    return static_cast<int>(h.n_enc);
 }
 
-// The persistent batch kernel alone, on a workspace planned already.
-int enqueue_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_cfg &c, cudaStream_t s) {
+// The persistent batch kernel alone, on a workspace planned already, of whose
+// messages n_enc encrypt.  No kernel runs before it that a fill could hide
+// behind, so a batch that only decrypts fills no encryption tables.
+int enqueue_batch_kernel(const aes_desc *desc, int n, int n_enc, void *ws, const aes_batch_cfg &c, cudaStream_t s) {
     if (n == 0) return AES_OK;
     if (n > AES_BATCH_MAX_DESCS) return AES_E_RANGE;
     int st = validate_batch_cfg(c);
     if (st != AES_OK) return st;
     int dev = 0;
     if (current_device(&dev) != AES_OK) return AES_E_CUDA;
-    return launch_batch_kernel(desc, n, ws, c, dev, s);
+    return launch_batch_kernel(desc, n, ws, c, n_enc > 0 ? kEncrypt : kDecrypt, dev, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -991,6 +1014,25 @@ int read_chunk_coverage(unsigned long long *once, unsigned long long *repeated, 
 #endif
 }
 
+// Debug build: the counts since the last call; clears them.
+int read_batch_counts(unsigned long long *fills, unsigned long long *counter) {
+#if defined(AESGB_BOUNDS_CHECK)
+    unsigned long long c[kCounts];
+    const unsigned long long zero[kCounts] = {};
+    if (cudaMemcpyFromSymbol(c, g_batch_counts, sizeof c) != cudaSuccess ||
+        cudaMemcpyToSymbol(g_batch_counts, zero, sizeof zero) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return AES_E_CUDA;
+    }
+    *fills = c[kCountFills];
+    *counter = c[kCountCounter];
+    return AES_OK;
+#else
+    *fills = *counter = 0;
+    return AES_E_CONFIG;
+#endif
+}
+
 }  // namespace aesgb
 
 using namespace aesgb;
@@ -1002,6 +1044,11 @@ size_t aes_batch_workspace_bytes(int n) { return n < 0 ? 0 : batch_ws_bytes(n); 
 int aes_debug_batch_coverage(unsigned long long *once, unsigned long long *repeated, unsigned long long *beyond) {
     if (!once || !repeated || !beyond) return AES_E_ARG;
     return read_chunk_coverage(once, repeated, beyond);
+}
+
+int aes_debug_batch_counts(unsigned long long *fills, unsigned long long *counter) {
+    if (!fills || !counter) return AES_E_ARG;
+    return read_batch_counts(fills, counter);
 }
 
 int aes_ecb_batch_ws(const aes_desc *desc_dev, int n, void *ws, size_t ws_bytes, int32_t *status_dev,

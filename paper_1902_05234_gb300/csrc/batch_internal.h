@@ -16,7 +16,7 @@ void batch_shutdown();
 
 // Host-side planning and the kernel alone (see batch.cu).
 size_t batch_plan_bytes(int n);  // the part of the workspace that a plan fills
-void plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host);
-int enqueue_batch_kernel(const aes_desc *desc, int n, void *ws, const aes_batch_cfg &c, cudaStream_t s);
+int plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host);
+int enqueue_batch_kernel(const aes_desc *desc, int n, int n_enc, void *ws, const aes_batch_cfg &c, cudaStream_t s);
 
 }  // namespace aesgb

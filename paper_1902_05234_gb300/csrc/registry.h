@@ -33,6 +33,7 @@ int bounds_violations_ct(unsigned long long *out);
 // batch.cu, debug build: exactly-once tags of the batch kernel's chunks (see
 // aes_debug_batch_coverage in aesgb.h); AES_E_CONFIG in the release build.
 int read_chunk_coverage(unsigned long long *once, unsigned long long *repeated, unsigned long long *beyond);
+int read_batch_counts(unsigned long long *fills, unsigned long long *counter);  // likewise (aes_debug_batch_counts)
 
 // Copy table `which` (0 te0, 1 td0, 2 S-box, 3 InvS) from the constant bank of
 // the encrypt module on the current device.  Returns a cudaError_t value.

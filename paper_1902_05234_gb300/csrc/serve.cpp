@@ -8,7 +8,7 @@
 //     a request that does not fit waits, and so do the ones behind it (FIFO);
 //   * packs the admitted requests (at most budget / slots bytes) into one
 //     batch as soon as one of the in-flight slots is free, plans it on the
-//     host (order and chunk prefix; the requests were validated at
+//     host (order and cost prefix; the requests were validated at
 //     submission) and launches it (descriptor and plan upload, the persistent
 //     batch kernel, completion event) on that slot's stream -- so requests
 //     that arrive while earlier batches run are
@@ -326,7 +326,7 @@ bool pack_locked(Server *s, Launch *L) {
 }
 
 // Plan the packed batch on the host and launch it on the slot's stream (mu
-// NOT held): the plan (message order, chunk prefix, zeroed counters) is built
+// NOT held): the plan (message order, cost prefix, zeroed counters) is built
 // here -- every request was validated at submission -- and uploaded with the
 // descriptors, so only the persistent kernel runs on the device.
 bool launch_unlocked(Server *s, const Launch &L) {
@@ -334,15 +334,15 @@ bool launch_unlocked(Server *s, const Launch &L) {
     Slot *sl = L.sl;
     const aes_batch_cfg cfg = batch_cfg_for(L.n);
     const size_t ws_off = plan_offset(L.n);
-    plan_on_host(sl->h_desc, L.n, cfg, reinterpret_cast<uint8_t *>(sl->h_desc) + ws_off);
+    const int n_enc = plan_on_host(sl->h_desc, L.n, cfg, reinterpret_cast<uint8_t *>(sl->h_desc) + ws_off);
     bool ok = cudaMemcpyAsync(sl->d_desc, sl->h_desc, ws_off + batch_plan_bytes(L.n), cudaMemcpyHostToDevice,
                               sl->stream) == cudaSuccess;
     ok = ok && (!L.wait_keys || cudaStreamWaitEvent(sl->stream, s->key_ev, 0) == cudaSuccess);
     // the batch that opens a busy period starts at the period's reference
     // event itself (interval start 0): one event record per launch fewer
     ok = ok && (!L.timed || cudaEventRecord(L.new_period ? s->ref : sl->t_start, sl->stream) == cudaSuccess);
-    ok = ok && enqueue_batch_kernel(sl->d_desc, L.n, reinterpret_cast<uint8_t *>(sl->d_desc) + ws_off, cfg,
-                                    sl->stream) == AES_OK;
+    ok = ok && enqueue_batch_kernel(sl->d_desc, L.n, n_enc, reinterpret_cast<uint8_t *>(sl->d_desc) + ws_off,
+                                    cfg, sl->stream) == AES_OK;
     ok = ok && (!L.timed || cudaEventRecord(sl->t_end, sl->stream) == cudaSuccess);
     ok = ok && cudaEventRecord(sl->ev, sl->stream) == cudaSuccess;
     if (!ok) (void)cudaGetLastError();

@@ -267,9 +267,25 @@ def run_server(aesgb, orc):
         for i in range(n):
             exp = orc.ecb(int(dirs[i]), keys[int(key_ids[i])], data[offs[i]:offs[i + 1]], nthreads=1)
             assert np.array_equal(got[offs[i]:offs[i + 1]], exp), ("served", i)
+        # requests that only decrypt: no kernel runs ahead of the batch kernel that
+        # a fill could hide behind, and every CTA fills its tables once
+        before = aesgb.aes_srv_stats(srv)["batches"]
+        aesgb.aes_debug_batch_counts()  # clear
+        st, tickets = aesgb.aes_srv_submit_many(srv, key_ids, np.ones(n, np.int32), ins, outs, sizes)
+        assert st == 0
+        aesgb.aes_srv_drain(srv, 60000)
+        status, _, _ = aesgb.aes_srv_results(srv, tickets, release=True)
+        assert np.all(status == 0)
+        fills, _ = aesgb.aes_debug_batch_counts()
+        batches = aesgb.aes_srv_stats(srv)["batches"] - before
+        assert fills == batches * aesgb.aes_device_sm_count(torch.cuda.current_device()), (fills, batches)
+        got = outp.cpu().numpy()
+        for i in range(n):
+            exp = orc.ecb(1, keys[int(key_ids[i])], data[offs[i]:offs[i + 1]], nthreads=1)
+            assert np.array_equal(got[offs[i]:offs[i + 1]], exp), ("served, decryption only", i)
     finally:
         aesgb.aes_srv_destroy(srv)
-    _report(aesgb, f"server ({n} requests, 8 keys)")
+    _report(aesgb, f"server ({2 * n} requests, 8 keys)")
 
 
 def main():

@@ -104,6 +104,9 @@ def test_debug_counter_is_debug_build_only(lib):
     c = [ctypes.c_ulonglong(7) for _ in range(3)]
     assert lib.aes_debug_batch_coverage(*[ctypes.byref(x) for x in c]) == -12
     assert [x.value for x in c] == [0, 0, 0]
+    c = [ctypes.c_ulonglong(7) for _ in range(2)]
+    assert lib.aes_debug_batch_counts(*[ctypes.byref(x) for x in c]) == -12
+    assert [x.value for x in c] == [0, 0]
 
 
 def test_fail_allocs_hook_arguments(lib):
