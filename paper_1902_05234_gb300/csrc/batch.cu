@@ -57,21 +57,19 @@ static_assert(offsetof(aes_desc, nblocks) == 24 && offsetof(aes_desc, nrounds) =
               "aes_desc field offsets");
 
 struct BatchHeader {
-    unsigned long long total_chunks;  // chunks of chunk_blocks blocks, all messages
-    unsigned long long enc_chunks;    // of the encryption messages
+    unsigned long long total_chunks;  // chunks of chunk_blocks blocks, all messages (debug build; else 0)
     unsigned long long enc_cost;      // costs [0, enc_cost) encrypt, [enc_cost, total_cost) decrypt
     unsigned long long total_cost;
     unsigned long long next[2];       // segment counters of the two phases (zeroed by the plan)
-    unsigned int n;
     unsigned int chunk_blocks;
-    unsigned int n_invalid;
     unsigned int n_enc;               // messages at positions [0, n_enc) encrypt
 };
 
 // What one plan CTA's descriptors add up to (count kernel -> place kernel).
 struct PlanTile {
-    unsigned long long cost[2], chunks[2];  // by direction
-    unsigned int n_enc, n_bad;
+    unsigned long long cost[2];  // by direction
+    unsigned long long chunks;   // debug build
+    unsigned int n_enc;
 };
 
 __host__ __device__ constexpr size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -165,32 +163,32 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 
 // Sums of the threads' tiles over the CTA, into *out (shared memory, zeroed).
 __device__ __forceinline__ void cta_sum(const PlanTile &t, PlanTile *out) {
-    const unsigned long long v[5] = {t.cost[0], t.cost[1], t.chunks[0], t.chunks[1],
-                                     static_cast<unsigned long long>(t.n_bad) << 32 | t.n_enc};
-    unsigned long long *dst[4] = {&out->cost[0], &out->cost[1], &out->chunks[0], &out->chunks[1]};
+    const bool lane0 = (threadIdx.x & 31) == 0;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const unsigned long long s = warp_sum(v[i]);
-        if ((threadIdx.x & 31) == 0 && s) {
-            if (i < 4) {
-                atomicAdd(dst[i], s);
-            } else {
-                atomicAdd(&out->n_enc, static_cast<unsigned int>(s));
-                atomicAdd(&out->n_bad, static_cast<unsigned int>(s >> 32));
-            }
-        }
+    for (int q = 0; q < 2; ++q) {
+        const unsigned long long s = warp_sum(t.cost[q]);
+        if (lane0 && s) atomicAdd(&out->cost[q], s);
     }
+    const unsigned int e = __reduce_add_sync(0xffffffffu, t.n_enc);
+    if (lane0 && e) atomicAdd(&out->n_enc, e);
+#if defined(AESGB_BOUNDS_CHECK)
+    const unsigned long long c = warp_sum(t.chunks);
+    if (lane0 && c) atomicAdd(&out->chunks, c);
+#endif
 }
 
 // One descriptor's share of its CTA's tile.  Invalid messages count as
 // encryptions without work, so they sit harmlessly in the first range.
 __device__ __forceinline__ PlanTile desc_tile(const aes_desc &d, int st, const PlanArgs &a) {
+    const bool ok = st == AES_OK, enc = !ok || d.dir == 0;
+    const unsigned long long cost = ok ? msg_cost(d.nblocks, d.nrounds, a.pass_shift) : 0ull;
     PlanTile t{};
-    const bool ok = st == AES_OK;
-    t.n_bad = !ok;
-    t.n_enc = !ok || d.dir == 0;
-    t.cost[t.n_enc ? 0 : 1] = ok ? msg_cost(d.nblocks, d.nrounds, a.pass_shift) : 0ull;
-    t.chunks[t.n_enc ? 0 : 1] = ok ? (d.nblocks + a.chunk_blocks - 1) / a.chunk_blocks : 0ull;
+    t.n_enc = enc;
+    t.cost[0] = enc ? cost : 0ull;
+    t.cost[1] = enc ? 0ull : cost;
+#if defined(AESGB_BOUNDS_CHECK)
+    t.chunks = ok ? (d.nblocks + a.chunk_blocks - 1) / a.chunk_blocks : 0ull;
+#endif
     return t;
 }
 
@@ -209,23 +207,23 @@ __global__ void __launch_bounds__(kPlanThreads, 1) batch_count_kernel(const __gr
     for (int i = first + static_cast<int>(threadIdx.x); i < a.n && i < first + a.per_cta; i += kPlanThreads) {
         const aes_desc d = a.desc[i];
         const PlanTile t = desc_tile(d, check_desc(d), a);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            sum.cost[q] += t.cost[q];
-            sum.chunks[q] += t.chunks[q];
-        }
+        sum.cost[0] += t.cost[0];
+        sum.cost[1] += t.cost[1];
+        sum.chunks += t.chunks;
         sum.n_enc += t.n_enc;
-        sum.n_bad += t.n_bad;
     }
     cta_sum(sum, &s_sum);
     __syncthreads();
     if (threadIdx.x == 0) ws_view(a.ws, a.n).tile[blockIdx.x] = s_sum;
 }
 
-// Statuses, partition positions and cost prefix.  A CTA starts from the tiles
-// of the CTAs before it (with one CTA, from nothing: its totals come from its
-// only scan).  Replaces one CTA that scanned all descriptors three times:
-// 20,000 descriptors took 87 us.
+// Statuses, partition positions and cost prefix.  Up to 1,024 descriptors this
+// kernel runs alone; above, two kernels, because a decryption's place takes the
+// totals of all encryptions first.  (One CTA that passes over the descriptors
+// twice instead: 2,048 messages of 64 B 20.6 -> 23.6 us with their batch, 4,096
+// 21.0 -> 33.2.)  A CTA starts from the tiles of the CTAs before it (with one
+// CTA, from nothing: its totals come from its only scan).  Replaces one CTA that
+// scanned all descriptors three times: 20,000 descriptors took 87 us.
 __global__ void __launch_bounds__(kPlanThreads, 1) batch_place_kernel(const __grid_constant__ PlanArgs a) {
     __shared__ PlanTile s_all, s_before;
     __shared__ unsigned long long s_cost[2][32];
@@ -305,13 +303,10 @@ __global__ void __launch_bounds__(kPlanThreads, 1) batch_place_kernel(const __gr
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         BatchHeader h{};
-        h.total_chunks = s_all.chunks[0] + s_all.chunks[1];
-        h.enc_chunks = s_all.chunks[0];
+        h.total_chunks = s_all.chunks;
         h.enc_cost = s_all.cost[0];
         h.total_cost = s_all.cost[0] + s_all.cost[1];
-        h.n = static_cast<unsigned int>(a.n);
         h.chunk_blocks = a.chunk_blocks;
-        h.n_invalid = s_all.n_bad;
         h.n_enc = s_all.n_enc;
         *v.hdr = h;
         v.start[a.n] = h.total_cost;
@@ -770,8 +765,8 @@ int enqueue_batch(const aes_desc *desc, int n, void *ws, size_t ws_bytes, int32_
 // Writes into a HOST buffer of batch_plan_bytes(n) bytes what the plan kernels
 // would write into that part of the workspace for these descriptors, which must
 // all be valid (check_desc): encryptions first in input order, then decryptions;
-// start[] the exclusive prefix of the costs; counters 0.  The chunk totals, which
-// the batch kernel does not read, stay 0.  Returns how many messages encrypt.
+// start[] the exclusive prefix of the costs; counters 0 (and no chunk total).
+// Returns how many messages encrypt.
 int plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_host) {
     const WsView v = ws_view(ws_host, n);
     const int shift = pass_shift(c);
@@ -793,7 +788,6 @@ int plan_on_host(const aes_desc *desc, int n, const aes_batch_cfg &c, void *ws_h
     }
     v.start[n] = run;
     h.total_cost = run;
-    h.n = static_cast<unsigned int>(n);
     h.chunk_blocks = batch_chunk_blocks(c);
     *v.hdr = h;
     return static_cast<int>(h.n_enc);

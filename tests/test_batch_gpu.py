@@ -219,6 +219,18 @@ def test_batch_graph_replay_and_library_workspace(orc):
     check_against_oracle(orc, b, b.output())
 
 
+def test_plan_sums_only_what_the_batch_kernel_reads():
+    """Chunk totals, the first field of the workspace's header, are the debug
+    build's: the release plan neither divides by the chunk nor sums them."""
+    torch = torch_cuda()
+    for n in (20, 1500):
+        lengths, keybits, dirs = small_mix(n, hi=1024, seed=15)
+        b = DeviceBatch(torch, lengths, keybits, dirs, seed=15)
+        ws, nbytes = b.workspace()
+        aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes)
+        assert int(ws[:8].cpu().numpy().view(np.uint64)[0]) == 0
+
+
 def test_batch_many_tiny_messages(orc):
     """20,000 messages of 16..256 bytes: the plan takes 20 CTAs of 1,024
     descriptors and the 32-ary search runs over 20,000 positions."""
