@@ -107,12 +107,11 @@ int aes_debug_bounds_violations(unsigned long long *count);
 int aes_test_fail_allocs(int skip, int count);
 
 /* Debug build only: exactly-once coverage of the batch kernel's work.
- * Each chunk (chunk_blocks consecutive blocks of one message, from its start)
- * adds one to its tag in the warp that takes its first pass, for chunk indices
- * below 65,536.
+ * Each pass that a warp takes is tagged in its chunk (chunk_blocks consecutive
+ * blocks of one message, from its start), for chunk indices below 65,536.
  * Returns, over all batch launches since the last call: *once the chunks
- * tagged exactly once, *repeated those tagged more than once, *beyond the
- * chunks whose index lies past the tags; then clears the tags.  After ONE
+ * with every pass tagged exactly once, *repeated those with one tagged more than
+ * once, *beyond the chunks whose index lies past the tags; then clears the tags.  After ONE
  * launch of T <= 65,536 chunks, *once == T and the others are 0.
  * AES_E_CONFIG with all three 0 in the release build.  DEVICE-synchronous. */
 int aes_debug_batch_coverage(unsigned long long *once, unsigned long long *repeated, unsigned long long *beyond);

@@ -353,11 +353,17 @@ __host__ __device__ constexpr uint32_t batch_table_bytes(int le, int ld) {
 }
 
 #if defined(AESGB_BOUNDS_CHECK)
-// Debug build: every chunk a warp takes adds one to its tag, so that after one
-// launch each of the T chunks must carry exactly 1 (aes_debug_batch_coverage
-// reads and clears the tags).  Chunks past the array are counted in bulk.
+// Debug build: every pass a warp takes sets its bit in its chunk's tag, so that
+// after one launch all passes of each of the T chunks must be set and none twice
+// (aes_debug_batch_coverage reads and clears the tags).  Segments are cut between
+// passes, also inside a chunk.  Chunks past the array are counted in bulk.
 constexpr unsigned int kTagChunks = 1u << 16;
-static __device__ unsigned int g_chunk_tag[kTagChunks];
+struct ChunkTag {
+    unsigned int seen[32];  // one bit per pass: a chunk has at most 1,024
+    unsigned int passes;    // how many it has, written by whoever takes one
+    unsigned int again;     // takings of a pass that was taken before
+};
+static __device__ ChunkTag g_chunk_tag[kTagChunks];
 static __device__ unsigned long long g_chunk_tag_beyond;
 #endif
 
@@ -488,18 +494,24 @@ __device__ __forceinline__ int find_message(const unsigned long long *start, int
 }
 
 #if defined(AESGB_BOUNDS_CHECK)
-// Debug build: tag the chunks of message `pos` whose first pass is one of
-// [j0, j1).  The chunks before the message's are counted over the partition.
-__device__ inline void tag_chunks(const BatchArgs &a, const WsView &v, int pos, unsigned long long j0,
-                                  unsigned long long j1, unsigned int pass_blocks) {
+// Debug build: tag passes [j0, j1) of message `pos`, which has `passes`.  The
+// chunks before the message's are counted over the partition.
+__device__ inline void tag_passes(const BatchArgs &a, const WsView &v, int pos, unsigned long long j0,
+                                  unsigned long long j1, unsigned long long passes, unsigned int pass_blocks) {
     const unsigned int cb = v.hdr->chunk_blocks, cp = cb / pass_blocks;
     unsigned long long before = 0;
     for (int q = 0; q < pos; ++q)
         if (v.start[q + 1] > v.start[q]) before += (a.desc[v.order[q]].nblocks + cb - 1) / cb;
-    for (unsigned long long k = (j0 + cp - 1) / cp; k * cp < j1; ++k) {
-        const unsigned long long c = before + k;
-        if (c < kTagChunks) atomicAdd(&g_chunk_tag[c], 1u);
-        else atomicAdd(&g_chunk_tag_beyond, 1ull);
+    for (unsigned long long j = j0; j < j1; ++j) {
+        const unsigned long long k = j / cp, c = before + k;
+        const unsigned int bit = static_cast<unsigned int>(j % cp);
+        if (c >= kTagChunks) {
+            if (bit == 0) atomicAdd(&g_chunk_tag_beyond, 1ull);
+            continue;
+        }
+        ChunkTag &t = g_chunk_tag[c];
+        t.passes = static_cast<unsigned int>(passes - k * cp < cp ? passes - k * cp : cp);
+        if (atomicOr(&t.seen[bit >> 5], 1u << (bit & 31)) >> (bit & 31) & 1u) atomicAdd(&t.again, 1u);
     }
 }
 #endif
@@ -557,7 +569,7 @@ __device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, 
                 e.count = static_cast<uint32_t>(end - first);
                 e.nr = d.nrounds;
 #if defined(AESGB_BOUNDS_CHECK)
-                if (take) tag_chunks(a, v, pos, j0, j1, kPass);
+                if (take) tag_passes(a, v, pos, j0, j1, passes, kPass);
 #endif
             }
             const unsigned int taken = __ballot_sync(0xffffffffu, take);
@@ -609,7 +621,11 @@ __device__ void batch_phase(const BatchArgs &a, const WsView &v, uint8_t *smem, 
 // worst of both: a warp that takes one more than the others ends late.  Equal
 // shares up to 1, 4, 8, 16 * most: 4,096 messages of up to 1 MiB 587 / 530 / 531
 // / 531 us, 1,000 of up to 4 MiB 522 / 472 / 472 / 472, 2,000 of them through the
-// server 1,259 / 1,198 / 1,196 / 1,200.
+// server 1,259 / 1,198 / 1,196 / 1,200.  Equal shares at every size instead lose
+// where SMs do not keep the same pace for milliseconds: 5.0 GB in 4,096 messages
+// 6,766 us from the counter and 6,830 in shares, 2.6 GB in 300 3,423 and 3,446,
+// 2.9 GB of decryption in 20 3,830 and 3,865, two streams of 2.6 GB 7,035 and
+// 7,105; one message of 1 GiB 1,601 and 1,597, of 5 GiB 6,867 and 6,875.
 __device__ __forceinline__ Segments cut(unsigned long long c, unsigned int W, unsigned int most) {
     Segments s;
     const unsigned long long share = (c + W - 1) / W;
@@ -975,11 +991,11 @@ int noalloc_scratch_ptr(int dev, void **out) {
     return AES_OK;
 }
 
-// Debug build: counts of chunks taken exactly once and more than once since
-// the last call, and of chunks past the tag array; clears the tags.
+// Debug build: counts of chunks with every pass taken exactly once, and with one
+// taken more than once, since the last call, and of chunks past the tag array; clears the tags.
 int read_chunk_coverage(unsigned long long *once, unsigned long long *repeated, unsigned long long *beyond) {
 #if defined(AESGB_BOUNDS_CHECK)
-    static unsigned int tags[kTagChunks];
+    static ChunkTag tags[kTagChunks];
     static std::mutex mu;
     std::lock_guard<std::mutex> lk(mu);
     const unsigned long long zero = 0;
@@ -990,9 +1006,11 @@ int read_chunk_coverage(unsigned long long *once, unsigned long long *repeated, 
     }
     *once = 0;
     *repeated = 0;
-    for (unsigned int i = 0; i < kTagChunks; ++i) {
-        *once += tags[i] == 1;
-        *repeated += tags[i] > 1;
+    for (const ChunkTag &t : tags) {
+        unsigned int seen = 0;
+        for (unsigned int w : t.seen) seen += static_cast<unsigned int>(__builtin_popcount(w));
+        *once += t.passes > 0 && seen == t.passes && t.again == 0;
+        *repeated += t.again > 0;
     }
     void *tag_addr = nullptr;
     if (cudaGetSymbolAddress(&tag_addr, g_chunk_tag) != cudaSuccess ||

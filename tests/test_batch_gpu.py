@@ -290,10 +290,9 @@ def test_library_workspace_batch_with_status(orc):
 def test_batch_plan_and_segment_edges(orc, n, invalid):
     """Sizes at which the plan takes one or several CTAs (1,024 descriptors
     each) and a warp one or several windows of 32 messages, with empty and
-    invalid messages in between (whole windows of them), one message that many
-    warps share, and each way a direction is cut: equal shares (the default
-    here), and long and short segments from the counter (few warps, one pass per
-    chunk)."""
+    invalid messages in between (whole windows of them), and one message that
+    many warps share.  All are cut into equal shares (the counter's segments:
+    test_batch_segments_from_the_counter)."""
     torch = torch_cuda()
     g = wl.rng(40 + n)
     lengths = 16 * g.integers(0, 70, size=n)
@@ -351,3 +350,27 @@ def test_batch_run_of_unused_descriptors_in_the_middle(orc, unused):
         check_against_oracle(orc, b, b.output(), skip=bad)
         times.append(stream_us(lambda s: aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes, stream=s), launches=20))
     assert times[0] <= 1.5 * times[1], times
+
+
+@pytest.mark.parametrize("inplace", [False, True])
+@pytest.mark.parametrize("nb, most", [(1, 200_000), (2, 400_000), (4, 800_000)])
+def test_batch_segments_from_the_counter(orc, nb, most, inplace):
+    """Above 192 * chunk_passes of cost per warp in a direction (passes times rounds
+    plus 6 for each message) the warps take long and short segments from the work
+    counter: few warps and one pass per chunk, in place too, where a pass taken
+    twice would show."""
+    torch = torch_cuda()
+    g = wl.rng(50 + nb)
+    n = 100
+    lengths = 16 * (g.integers(1, most, size=n) // 16)
+    lengths[[3, 40, 77]] = (16, 0, 16 * (32 * nb * 600 + 1))
+    keybits, dirs = g.choice(np.array([128, 192, 256]), size=n), g.integers(0, 2, size=n)
+    b = DeviceBatch(torch, lengths, keybits, dirs, seed=51, inplace=inplace)
+    cfg = aesgb.make_batch_cfg(32, nb, 1, 1, aesgb.LAYOUT_R4, aesgb.LAYOUT_R4)
+    cost = np.where(b.lengths > 0, -(-b.lengths // (512 * nb)) * b.nrounds + 6, 0)
+    warps = aesgb.aes_device_sm_count(torch.cuda.current_device())
+    for d in (0, 1):
+        assert int(cost[b.dirs == d].sum()) > 1.2 * 192 * warps, "equal shares"
+    ws, nbytes = b.workspace()
+    aesgb.aes_ecb_batch_ws(b.desc_dev, n, ws, nbytes, cfg=cfg)
+    check_against_oracle(orc, b, b.output())

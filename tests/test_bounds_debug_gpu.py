@@ -204,7 +204,7 @@ def run_batch(aesgb, orc):
     exp = np.concatenate([e for _, e in sorted(expected(b).items())])
     ws, nbytes = b.workspace()
     ncfg = 0
-    pairs = [(aesgb.LAYOUT_R4, aesgb.LAYOUT_R2, (1, 2, 4)), (aesgb.LAYOUT_R4, aesgb.LAYOUT_R4, (1, 2)),
+    pairs = [(aesgb.LAYOUT_R4, aesgb.LAYOUT_R2, (1, 2, 4)), (aesgb.LAYOUT_R4, aesgb.LAYOUT_R4, (1, 2, 4)),
              (aesgb.LAYOUT_R2, aesgb.LAYOUT_R2, (1, 2)), (aesgb.LAYOUT_R1, aesgb.LAYOUT_R1, (1, 2))]
     cfgs = [aesgb.make_batch_cfg(threads, nb, passes, 1, le, ld)
             for le, ld, nbs in pairs for nb in nbs for threads in (64, 512) for passes in (1, 5)]
@@ -214,6 +214,18 @@ def run_batch(aesgb, orc):
         tagged += check_coverage(n_chunks(b, cfg), ws)
         assert np.array_equal(b.output(), exp), ("batch cfg", repr(cfg))
         ncfg += 1
+    # segments from the work counter: more than 192 of cost per warp and direction
+    lengths, keybits, dirs = mix(60, 2 << 20, 344)
+    c = DeviceBatch(torch, lengths, keybits, dirs, seed=345, inplace=True)
+    cexp = np.concatenate([e for _, e in sorted(expected(c).items())])
+    cws, cbytes = c.workspace()
+    aesgb.aes_debug_batch_counts()  # clear
+    cfg = aesgb.make_batch_cfg(32, 1, 1, 1, aesgb.LAYOUT_R4, aesgb.LAYOUT_R4)
+    aesgb.aes_ecb_batch_ws(c.desc_dev, c.n, cws, cbytes, cfg=cfg)
+    tagged += check_coverage(n_chunks(c, cfg), cws)
+    assert np.array_equal(c.output(), cexp), "segments from the counter"
+    assert aesgb.aes_debug_batch_counts()[1] > 0
+
     default = n_chunks(b, aesgb.aes_batch_get_cfg(b.n))
     b.out_dev.fill_(0x5A)
     aesgb.aes_ecb_batch(b.desc_dev, b.n)
