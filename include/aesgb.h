@@ -369,7 +369,8 @@ int aes_ecb_host(int dir, const uint32_t *rk, int nrounds, const uint8_t *host_i
  * page-locked and mapped for the device (cudaHostAlloc / cudaHostRegister with
  * mapping, or torch's pin_memory), else AES_E_ARG.  The kernel reads and
  * writes them over the host link itself -- no staging buffer, no copies, no
- * internal streams; throughput is that of the link.  Same cipher, rk and
+ * internal streams; throughput is that of the link.  The launch shape is the
+ * one for host memory at that size, whatever the tuner chose on device buffers.  Same cipher, rk and
  * overlap rules as aes_ecb_encrypt/decrypt; asynchronous on `stream`.  The
  * buffers must hold nblocks*16 bytes (only their first bytes are checked). */
 int aes_ecb_host_direct(int dir, const uint32_t *rk, int nrounds, const uint8_t *host_in, uint8_t *host_out,

@@ -157,7 +157,7 @@ int launch_pdl(const void *fn, int grid, int threads, uint32_t smem, void **para
 }
 
 int launch_ecb(int dir, const uint32_t *rk, int nr, const uint8_t *in, uint8_t *out, size_t nblocks,
-               const aes_launch_cfg &c, void *stream) {
+               const aes_launch_cfg &c, void *stream, bool host_memory) {
     const void *fn = ecb_kernel_ptr(dir, nr, c);
     if (!fn) return AES_E_CONFIG;
     int dev = 0;
@@ -172,6 +172,8 @@ int launch_ecb(int dir, const uint32_t *rk, int nr, const uint8_t *in, uint8_t *
     args.out = reinterpret_cast<uint4 *>(out);
     args.nblocks = nblocks;
     order_round_keys(dir, rk, nr, &args.rk);
+    args.warp_stride = host_memory ? 1u : static_cast<uint32_t>(grid);
+    args.cta_stride = host_memory ? static_cast<uint32_t>(c.threads / 32) : 1u;
     uint32_t extra_tx = 0;  // the TMA-staged kernel's second parameter
     void *params[] = {&args, &extra_tx};
     return launch_pdl(fn, grid, c.threads, smem, params, stream);

@@ -33,8 +33,9 @@ int validate_cfg(const aes_launch_cfg &c);
 // never more than the work needs.
 int persistent_grid(const void *fn, int dev, const aes_launch_cfg &c, uint32_t smem,
                     unsigned long long work_items_per_cta, unsigned long long total_items, int *grid);
+// host_memory: the buffers are page-locked host memory, at their device addresses.
 int launch_ecb(int dir, const uint32_t *rk, int nr, const uint8_t *in, uint8_t *out, size_t nblocks,
-               const aes_launch_cfg &c, void *stream);
+               const aes_launch_cfg &c, void *stream, bool host_memory = false);
 
 // keysched.cpp
 int expand_key_host(int keybits, const uint8_t *key, uint32_t *rk_enc, uint32_t *rk_dec);

@@ -8,6 +8,8 @@
 // Ordering is carried by events recorded per slot; the caller's stream is
 // joined at the start (earlier work on it finishes first) and at the end (it
 // waits for the last copy-out).
+//
+// aes_ecb_host_direct launches the kernel on the host buffers themselves.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -64,6 +66,24 @@ void destroy_res(HostIoRes &r) {
     r.s_in = r.s_run = r.s_out = nullptr;
     r.ev_begin = nullptr;
     r.ready = false;
+}
+
+// Launch shape over host memory, both directions.  The link bounds it (343 GB/s
+// both ways), and the shapes that suit HBM do not: a few warps per SM are enough
+// for the link's latency, and more of them only spread its requests.  R4 tables,
+// one CTA per SM, one block per thread, 256 threads below 8,192 blocks per SM
+// (19 MiB), 512 below 32,768, 1,024 above.  The untuned HBM shapes / this (us):
+//   AES-128 encryption  1 MiB 9.6 / 8.5, 4 MiB 35.8 / 28.6, 16 MiB 109.9 / 104.9,
+//                       64 MiB 407.3 / 404.2, 256 MiB 1,612 / 1,592
+//   AES-256 decryption  1 MiB 9.7 / 8.8, 4 MiB 36.1 / 28.6, 16 MiB 110.8 / 105.8,
+//                       64 MiB 430.8 / 411.8, 1 GiB 6,493 / 6,438
+// and 256 / 512 / 1,024 threads, AES-256 encryption: 16 MiB 105.8 / 106.5 / 110.7,
+// 64 MiB - / 407.0 / 408.1, 120 MiB - / 760.6 / 755.1.  Tuned entries were timed
+// on HBM and do not count here.
+aes_launch_cfg host_memory_cfg(int dev, size_t nblocks) {
+    const int sms = sm_count(dev);
+    const size_t per_sm = nblocks / static_cast<size_t>(sms > 0 ? sms : 152);
+    return aes_launch_cfg{per_sm < 8192 ? 256 : per_sm < 32768 ? 512 : 1024, 1, AES_LAYOUT_R4, 1};
 }
 
 }  // namespace
@@ -162,7 +182,8 @@ extern "C" int aes_ecb_host_direct(int dir, const uint32_t *rk, int nrounds, con
         if (a.type != cudaMemoryTypeHost || a.devicePointer == nullptr) return AES_E_ARG;
         dev_ptr[i] = a.devicePointer;
     }
-    const aes_launch_cfg cfg = tuned_or_default_cfg(dir, nrounds, nblocks);
+    int dev = 0;
+    if (current_device(&dev) != AES_OK) return AES_E_CUDA;
     return launch_ecb(dir, rk, nrounds, static_cast<const uint8_t *>(dev_ptr[0]), static_cast<uint8_t *>(dev_ptr[1]),
-                      nblocks, cfg, stream);
+                      nblocks, host_memory_cfg(dev, nblocks), stream, true);
 }

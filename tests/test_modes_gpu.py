@@ -106,6 +106,43 @@ def test_ecb_host_direct(orc):
     assert e.value.status == -1
 
 
+@pytest.mark.parametrize("per_sm", [1, 8192, 32768])
+def test_ecb_host_direct_launch_shapes(orc, per_sm):
+    """Over host memory the threads per CTA change at 8,192 and 32,768 blocks per SM
+    and units are numbered CTA by CTA: both sides of each line, the first and last
+    blocks against the oracle and all of them against device buffers."""
+    torch = torch_cuda()
+    edge = aesgb.aes_device_sm_count(torch.cuda.current_device()) * per_sm
+    enc, dec, nr = aesgb.aes_expand_key(256, wl.random_key(256, 102).tobytes())
+    for n in (edge - 1, edge + 33):
+        x = torch.empty(16 * n, dtype=torch.uint8, device="cuda").random_(0, 256)
+        h_in, h_out = x.cpu().pin_memory(), torch.zeros(16 * n, dtype=torch.uint8).pin_memory()
+        for direction, rk in ((0, enc), (1, dec)):
+            y = torch.empty_like(x)
+            aesgb.aes_ecb_crypt_cfg(direction, rk, nr, x, y, n, aesgb.make_cfg(256, 1, aesgb.LAYOUT_R2, 0))
+            aesgb.aes_ecb_host_direct(direction, rk, nr, h_in, h_out, n)
+            torch.cuda.synchronize()
+            assert torch.equal(h_out, y.cpu()), (n, direction)
+            for part in (slice(0, 4096), slice(max(0, 16 * n - 4096), 16 * n)):
+                exp = orc.ecb(direction, wl.random_key(256, 102).tobytes(), h_in.numpy()[part])
+                assert np.array_equal(h_out.numpy()[part], exp), (n, direction, part)
+
+
+def test_ecb_host_direct_shape_suits_the_link():
+    """4 MiB of host memory: 256 threads per SM measure 0.80 of the 1,024 that
+    device memory takes, both directions."""
+    torch = torch_cuda()
+    enc, dec, nr = aesgb.aes_expand_key(128, wl.random_key(128, 103).tobytes())
+    n = 1 << 18
+    h_in = torch.zeros(16 * n, dtype=torch.uint8).pin_memory()
+    h_out = torch.zeros(16 * n, dtype=torch.uint8).pin_memory()
+    for direction, rk in ((0, enc), (1, dec)):
+        cfg = aesgb.make_cfg(1024, 1, aesgb.LAYOUT_R4, 1)
+        wide = stream_us(lambda s: aesgb.aes_ecb_crypt_cfg(direction, rk, nr, h_in, h_out, n, cfg, s), launches=20)
+        direct = stream_us(lambda s: aesgb.aes_ecb_host_direct(direction, rk, nr, h_in, h_out, n, s), launches=20)
+        assert direct <= 0.92 * wide, (direction, direct, wide)
+
+
 @pytest.mark.parametrize("keybits", [128, 192, 256])
 def test_cfb_decrypt_matches_oracle(orc, keybits):
     """CFB decryption (full-block CFB; the forward cipher on the previous
