@@ -626,7 +626,8 @@ def aes_batch_graph_destroy(graph: int) -> None:
 
 
 def make_batch_cfg(threads=512, blocks_per_thread=1, chunk_passes=32, ctas_per_sm=1, layout_enc=LAYOUT_R4,
-                   layout_dec=LAYOUT_R2) -> aes_batch_cfg:
+                   layout_dec=LAYOUT_R4) -> aes_batch_cfg:
+    """A batch configuration; the defaults are those of the untuned library."""
     return aes_batch_cfg(int(threads), int(blocks_per_thread), int(chunk_passes), int(ctas_per_sm),
                          int(layout_enc), int(layout_dec))
 

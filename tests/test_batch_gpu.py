@@ -137,12 +137,13 @@ def batch_cfgs():
     for nb in (1, 2, 4):
         for threads in (64, 256, 512):
             for passes in (1, 3, 8):
-                out.append(aesgb.make_batch_cfg(threads, nb, passes, 1))
+                out.append(aesgb.make_batch_cfg(threads, nb, passes, 1, *LAYOUT_PAIRS[0]))
     for le, ld in LAYOUT_PAIRS[1:]:                  # the other table layouts of the two phases
         for nb in (1, 2):
             for threads in (64, 512):
                 for passes in (1, 8):
                     out.append(aesgb.make_batch_cfg(threads, nb, passes, 1, le, ld))
+    out.append(aesgb.make_batch_cfg(512, 4, 3, 1, *LAYOUT_PAIRS[1]))
     return out
 
 

@@ -218,6 +218,11 @@ def test_tune_cache_file_roundtrip(tmp_path):
         aesgb.aes_tune_clear()
 
 
+def test_make_batch_cfg_defaults_are_the_librarys():
+    aesgb.aes_tune_clear()
+    assert repr(aesgb.make_batch_cfg()) == repr(aesgb.aes_batch_get_cfg(4096))
+
+
 def test_batch_default_cfg_valid():
     c = aesgb.aes_batch_get_cfg(4096)
     assert c.threads <= 512 and c.blocks_per_thread in (1, 2, 4) and c.chunk_passes >= 1
