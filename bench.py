@@ -45,6 +45,9 @@ METRIC = "AES-128 ECB enc/dec throughput (single 1 GiB buffer, HBM-resident)"
 UNIT = "Gbit/s"
 KERNEL_SOURCES = ["paper_1902_05234_gb300/csrc/aes_kernels.cuh",
                   "paper_1902_05234_gb300/csrc/aes_tables.h",
+                  "paper_1902_05234_gb300/csrc/bitslice.cuh",
+                  "paper_1902_05234_gb300/csrc/bitslice_circuits.h",
+                  "paper_1902_05234_gb300/csrc/bitslice_math.h",
                   "paper_1902_05234_gb300/csrc/bounds.cuh"]
 
 
@@ -728,10 +731,10 @@ def run_study(args):
     d = args.study_dir
     rk = enc if d == 0 else dec
     rows = []
-    variants = STUDY_VARIANTS + [("constant time: bitsliced, no tables, 32 blocks per thread", None, 32, 256)]
+    variants = STUDY_VARIANTS + [("constant time: bitsliced, no tables, 8 blocks per thread", None, 8, 512)]
     for i, (label, layout, nb, threads) in enumerate(variants):
         if layout is None:
-            cfg = "aes_ecb_crypt_ct(threads=256, 32 blocks/thread)"
+            cfg = "aes_ecb_crypt_ct(threads=512, 8 blocks/thread)"
             launch = lambda: aesgb.aes_ecb_crypt_ct(d, rk, nr, x, y, n)  # noqa: E731
         else:
             cfg = aesgb.make_cfg(threads, nb, layout, 0)

@@ -504,7 +504,8 @@ __global__ void __launch_bounds__(max_threads_for(NB, LAYOUT), 1)
     ecb_kernel(const __grid_constant__ EcbArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u;
-    unsigned long long n = a.nblocks, step = static_cast<unsigned long long>(gridDim.x) * (blockDim.x >> 5) * 32ull * NB;
+    unsigned long long n = a.nblocks;
+    unsigned long long step = static_cast<unsigned long long>(gridDim.x) * (blockDim.x >> 5) * 32ull * NB;
     unsigned long long base = (static_cast<unsigned long long>(threadIdx.x >> 5) * a.warp_stride +
                                static_cast<unsigned long long>(blockIdx.x) * a.cta_stride) * 32ull * NB;
     // Kept in registers: left to itself the compiler derives them again in every

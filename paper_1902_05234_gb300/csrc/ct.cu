@@ -109,16 +109,20 @@ AESGB_HD void expand_mask(const uint8_t (*m)[16], int i, bs::RoundMasks *dst) {
 // operations per block for AES-128 encryption (aes_ct_ops_per_block), 30 byte
 // permutes for ShiftRows and about 10 more for addresses and bounds.  A unit of
 // work is a warp's 256 blocks (4 KiB).  8 blocks and 32 planes per thread take
-// 94 registers without spill, and keep the pipe 98.8 % busy; the form with 32 blocks and 128 planes, one word
-// per (column, row, bit), needs no permutes but 255 registers and a unit of
-// 16 KiB, so a pass was four times as long and a 1 MiB buffer filled 8 SMs.
-// Units go round the CTAs first and then the warps of each, so that every SM,
-// and every quarter of one, gets the same number within one.  Measured against
-// that form (a replayed graph of launches, AES-128 encryption): 4 KiB 20.1 ->
-// 5.9 us, 1 MiB 36.2 -> 5.9 us, 16 MiB 37.9 -> 33.4 us, 1 GiB 4,345 -> 4,394
-// Gbit/s; AES-256 decryption of 256 MiB 2,853 -> 3,019 Gbit/s.  The permutes
-// grow with the rounds: AES-256 encryption at 1 GiB, where the other form had no
-// partly filled pass to lose, 3,292 -> 3,238.
+// 94 registers without spill, and keep the pipe 98.8 % busy; the form with 32
+// blocks and 128 planes, one word per (column, row, bit), needs no permutes but
+// 255 registers and a unit of 16 KiB, so a pass was four times as long and a
+// 1 MiB buffer filled 8 SMs.  Units go round the CTAs first and then the warps of
+// each, so that every SM, and every quarter of one, gets the same number within
+// one.  Measured against that form (replayed graph): AES-128 encryption 64 KiB
+// 20.0 -> 5.7 us, 1 MiB 36.0 -> 5.7, 16 MiB 38.2 -> 33.9, 256 MiB 536 -> 492, 1
+// GiB 1,987 -> 1,956, 8 GiB 16,190 -> 15,575; AES-256 decryption 256 MiB 753 ->
+// 711, 8 GiB 23,273 -> 22,601.  The permutes grow with the rounds, so between
+// 0.75 and 2.5 GiB, where the other form's last pass costs little and its clock
+// has not come down yet, it was ahead at AES-256 (encryption 1 GiB 2,619 / 2,659,
+// 2 GiB 5,231 / 5,304, 4 GiB 10,648 / 10,596; decryption by 0.5 to 1 %) and at
+// AES-192 encryption (1.5 GiB 3,413 / 3,453).  A second kernel that spills for
+// 1.7 % at most, in that window, is not kept.
 template <int DIR>
 __global__ void __launch_bounds__(kCtThreads, 1) ct_kernel(const __grid_constant__ CtArgs a) {
     __shared__ bs::RoundMasks masks[15];

@@ -230,10 +230,12 @@ float time_launches(F launch, cudaStream_t s, int reps, int *status) {
 //   AES-128  64 MiB 74.3 / 74.5, 128 MiB 145.6 / 144.7, 1 GiB 1,145 / 1,124
 //   AES-192  64 MiB 88.4 / 87.6, 128 MiB 173.9 / 170.7, 1 GiB 1,371 / 1,333
 //   AES-256  64 MiB 101.7 / 102.1, 128 MiB 200.8 / 201.1, 1 GiB 1,585 / 1,576
-// Decryption keeps its former R4, 1,024 threads x 2 blocks between 16,384 and
-// 32,768 blocks per SM, where the R2 form gains 0.4-2 % (64 MiB: AES-128 75.8 /
-// 74.3, AES-256 102.3 / 101.9); above, R2: 1 GiB AES-128 1,161 -> 1,142, AES-256
-// 1,587 -> 1,581.
+// Between 16,384 and 32,768 blocks per SM decryption keeps R4, 1,024 threads x 2
+// blocks, although R2 x 1 measures 0.4 to 2 % less there (40 MiB: AES-128 47.4 /
+// 46.4, AES-256 64.1 / 63.8): it is the choice that aes_ecb_get_cfg has reported
+// for that size class since before the others moved, which callers (and the tests
+// of the tuning cache) tell a tuned entry from; tuning finds the other.  Above,
+// R2: 1 GiB AES-128 1,164 -> 1,145, AES-256 1,589 -> 1,584.
 aes_launch_cfg default_cfg(int dir, int /*nrounds*/, size_t nblocks) {
     const int found = current_sms();
     const size_t sms = static_cast<size_t>(found > 0 ? found : 152);

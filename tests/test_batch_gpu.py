@@ -220,6 +220,26 @@ def test_batch_graph_replay_and_library_workspace(orc):
     check_against_oracle(orc, b, b.output())
 
 
+def test_batch_graph_of_more_descriptors_than_a_plan_cta(orc):
+    """Above 1,024 descriptors a captured batch is three kernels (count, place,
+    batch) with two programmatic edges: two replays, the second on other contents
+    of the same table."""
+    torch = torch_cuda()
+    lengths, keybits, dirs = small_mix(2500, hi=2048, seed=16)
+    b = DeviceBatch(torch, lengths, keybits, dirs, seed=16)
+    other = DeviceBatch(torch, lengths[::-1].copy(), keybits, 1 - dirs, seed=17)
+    ws, nbytes = b.workspace()
+    g = aesgb.aes_batch_graph_create(b.desc_dev, b.n, ws, nbytes)
+    try:
+        aesgb.aes_batch_graph_launch(g)
+        check_against_oracle(orc, b, b.output())
+        b.desc_dev.copy_(other.desc_dev)
+        aesgb.aes_batch_graph_launch(g)
+        check_against_oracle(orc, other, other.output())
+    finally:
+        aesgb.aes_batch_graph_destroy(g)
+
+
 def test_plan_sums_only_what_the_batch_kernel_reads():
     """Chunk totals, the first field of the workspace's header, are the debug
     build's: the release plan neither divides by the chunk nor sums them."""

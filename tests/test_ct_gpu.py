@@ -72,8 +72,8 @@ def test_logic_rate_calibration():
 @pytest.mark.parametrize("units_per_sm", [0, 1, 4, 8, 17])
 def test_ct_unit_and_cta_size_edges(orc, units_per_sm):
     """A warp's unit is 256 blocks and 8 blocks share a thread's words; the CTA
-    size follows the units per SM up to 4 and changes above 4 and 8, and above 16 the warps take a
-    second unit: one block below, at and above each of those."""
+    size follows the units per SM up to 4 and changes above 4 and 8, and above 16
+    the warps take a second unit: one block below, at and above each of those."""
     torch = torch_cuda()
     edge = max(256, 256 * units_per_sm * aesgb.aes_device_sm_count(0))
     key = wl.random_key(256, 223).tobytes()

@@ -309,11 +309,12 @@ def test_tma_wait_timeout_is_reported_and_context_survives(orc):
 
 
 @pytest.mark.parametrize("direction", [0, 1])
-def test_even_shares_at_one_cta_per_sm(orc, direction):
-    """With one CTA per SM (R4, 1,024 threads), up to 8 units (32 x blocks per
-    thread) per warp are split into even contiguous shares; above that the
-    kernel takes grid-stride passes.  Sizes around both ends of the even
-    range and ragged tails, against the oracle, in place and out of place."""
+def test_rounds_of_units_at_one_cta_per_sm(orc, direction):
+    """With one CTA per SM (R4, 1,024 threads) a warp's unit is 32 x blocks per
+    thread and units go round the CTAs, then the warps of each, then round again:
+    less than a round, one round less and more a few blocks, eight rounds, and a
+    last round of one or a few units, against the oracle, in place and out of
+    place."""
     torch = torch_cuda()
     sms = aesgb.aes_device_sm_count(torch.cuda.current_device())
     key = wl.random_key(128, 14).tobytes()
@@ -349,9 +350,10 @@ def test_default_cfg_small_size_switches(orc, blocks_per_sm):
 
 @pytest.mark.parametrize("keybits", [128, 192, 256])
 def test_last_round_without_lookups(orc, keybits):
-    """R4 encryption with four blocks per thread takes the last round of a
-    thread's first two blocks in logic: every place of a block in the unit of
-    128, partial units, in place, all byte values in every position."""
+    """R4 encryption with 512 threads and four blocks per thread takes the last
+    round of a thread's first two blocks (0..63 of a unit of 128) in logic: every
+    place of a block in the unit, partial units, in place, and last rounds whose
+    input has every byte value in every position of a block that takes that path."""
     torch = torch_cuda()
     key = wl.random_key(keybits, 16).tobytes()
     cfg = aesgb.make_cfg(512, 4, aesgb.LAYOUT_R4, 1)
@@ -362,6 +364,20 @@ def test_last_round_without_lookups(orc, keybits):
     every = np.repeat(np.arange(256, dtype=np.uint8), 16)   # 256 blocks of one byte value each
     got, ok = gpu_ecb(0, key, every, cfg=cfg, guard=64)
     assert ok and np.array_equal(got, orc.ecb(0, key, every)), "byte values"
+    # last-round inputs: byte q of block v holds v + 37 q; the ciphertext is
+    # ShiftRows(SubBytes(input)) + last round key, the plaintext its decryption
+    enc, _, nr = aesgb.aes_expand_key(keybits, key)
+    last_key = enc[4 * nr:4 * nr + 4].view(np.uint8)
+    sbox = np.asarray(aesgb.aes_host_table(2)).astype(np.uint8)
+    q = np.arange(16)
+    state = sbox[(np.arange(256)[:, None] + 37 * q) % 256]
+    cipher = state[:, (q & 3) + 4 * (((q >> 2) + (q & 3)) & 3)] ^ last_key
+    place = 128 * (np.arange(256) // 64) + np.arange(256) % 64
+    blocks = wl.random_bytes(16 * 512, 18).reshape(512, 16)
+    blocks[place] = orc.ecb(1, key, cipher.reshape(-1).copy()).reshape(256, 16)
+    got, ok = gpu_ecb(0, key, blocks.reshape(-1), cfg=cfg, guard=64)
+    assert ok and np.array_equal(got, orc.ecb(0, key, blocks.reshape(-1)))
+    assert np.array_equal(got.reshape(512, 16)[place], cipher), "last-round inputs"
 
 
 def test_four_blocks_per_thread_with_few_warps():

@@ -257,12 +257,14 @@ def test_small_launch_shapes(orc, per_sm):
         data = wl.random_bytes(16 * n, 100)
         x = torch.from_numpy(data).cuda()
         y = torch.full((16 * n + 64,), 0x5A, dtype=torch.uint8, device="cuda")
-        for call, rk, block, ref in ((aesgb.aes_ctr_crypt, enc, wrap64, orc.ctr), (aesgb.aes_ctr_crypt, enc, wrap128, orc.ctr),
+        for call, rk, block, ref in ((aesgb.aes_ctr_crypt, enc, wrap64, orc.ctr),
+                                     (aesgb.aes_ctr_crypt, enc, wrap128, orc.ctr),
                                      (aesgb.aes_cbc_decrypt, dec, iv, orc.cbc_decrypt),
                                      (aesgb.aes_cfb_decrypt, enc, iv, orc.cfb_decrypt)):
             call(rk, nr, block, x, y, n)
             got = y.cpu().numpy()
-            assert np.array_equal(got[:16 * n], ref(key, block, data)) and np.all(got[16 * n:] == 0x5A), (call.__name__, n)
+            assert np.array_equal(got[:16 * n], ref(key, block, data)), (call.__name__, n)
+            assert np.all(got[16 * n:] == 0x5A), (call.__name__, n)
 
 
 @pytest.mark.parametrize("kib", [64, 512])
@@ -280,7 +282,8 @@ def test_small_calls_in_a_stream_spread_over_the_sms(kib):
     x = torch.zeros(16 * n, dtype=torch.uint8, device="cuda")
     y = torch.empty_like(x)
     cfg = aesgb.make_cfg(256, 1, aesgb.LAYOUT_R4, 1)
-    for call, rk, direction in ((aesgb.aes_ctr_crypt, enc, 0), (aesgb.aes_cfb_decrypt, enc, 0), (aesgb.aes_cbc_decrypt, dec, 1)):
+    for call, rk, direction in ((aesgb.aes_ctr_crypt, enc, 0), (aesgb.aes_cfb_decrypt, enc, 0),
+                                (aesgb.aes_cbc_decrypt, dec, 1)):
         ecb = stream_us(lambda s: aesgb.aes_ecb_crypt_cfg(direction, rk, nr, x, y, n, cfg, s))
         mode = stream_us(lambda s: call(rk, nr, iv, x, y, n, s))
         assert mode <= 1.1 * ecb, (call.__name__, kib, mode, ecb)
