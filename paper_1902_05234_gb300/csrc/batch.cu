@@ -656,10 +656,13 @@ constexpr int kBatchMaxThreads = 512;  // up to 128 registers: round keys live i
 // first blocks), which is why the next message's are always under way, and why
 // a batch that gives a warp up to 16 chunks is cut into equal shares instead of
 // whole chunks.  Against one chunk of one message at a time, found by
-// a search each, behind a one-CTA plan: 20,000 messages of 16 B to 16 KiB 217 ->
-// 97 us (plan 87 -> about 9), 2,000 of them 64 -> 31, 20 of them 38 -> 10.5;
-// 2,000 of up to 4 MiB 908 -> 884 us (kernel and plan), 4,096 of up to 16 MiB
-// (5.2 GB) 6,669 -> 6,650.  With 512 threads and the 44 to 60 key words in registers a
+// a search each, behind a one-CTA plan (replayed graph, plan and kernel): 20,000
+// messages of 16 B to 16 KiB 221 -> 92.6 us, 2,000 of them 70 -> 25.6, 20 of them
+// 26 -> 8.5; 4,096 of up to 1 MiB 582 -> 539, 2,000 of up to 4 MiB 1,057 -> 1,035
+// (745 MiB); 4,096 of up to 16 MiB the same within 0.4 %, decryption alone 0.3 %
+// slower, and one decryption of 5 GiB 1.2 % (R4 tables).  A batch without work, the
+// plan and an idle kernel: 4.2 us with one descriptor, 6.9 with 1,024, 9.0 with
+// 1,025, 9.3 with 20,000, 10.0 with 100,000.  With 512 threads and the 44 to 60 key words in registers a
 // thread has one block in flight; two measured 20 % slower.
 template <int NB, int LE, int LD>
 __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_kernel(const __grid_constant__ BatchArgs a) {
